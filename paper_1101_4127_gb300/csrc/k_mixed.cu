@@ -435,56 +435,66 @@ __device__ __forceinline__ long long cell_attenuate(float seg, float dl, float4 
 // Where a walk reads absorbers and adds deposits: the grid in global memory
 // (gathers through L1, deposits reduced in L2) ...
 //
-// The four int64 deposits of a crossing are one 32-byte record, so they go
-// to L2 as one bulk reduction (cp.reduce.async.bulk .add.u64) from a 32-byte
-// slot of shared memory per thread instead of four separate reductions.
-// Two slots alternate: a slot is rewritten only after the bulk operation
-// issued from it two crossings earlier has read it.  Integer sums do not
-// depend on their order, so the deposits are the same bits either way.
-// Without a slot (stage == nullptr: more than kStageThreads threads, or a
-// deposit array not aligned to 16 bytes) the thread uses plain reductions.
-constexpr int kStageThreads = 256;
+// The four int64 deposits of a crossing are one 32-byte record (one sector).
+// A warp sends the records of its lanes together: every lane stores its
+// record to the warp's staging area in shared memory, and the warp then walks
+// the 32 records in four steps of eight, four lanes to a record, each lane
+// adding one of its int64 values with one reduction.  The four lanes of a
+// record address one sector, so a step is one warp instruction of eight
+// sectors.  Sending a record per lane takes 32 sectors per instruction (four
+// plain reductions) or, as a 32-byte bulk reduction, one issue per lane with
+// its addresses moved to uniform registers (about 8.6 warp instructions per
+// record).  Integer sums do not depend on their order, so the deposits are
+// the same bits in every form.
+constexpr int kMaxWarps = 8;             // 256 threads: the kernels' launch bound
+constexpr int kStageHalf = 576;          // second half-records: 512 bytes on, and 64 more so that the
+                                         // read below touches every bank once per half warp
+constexpr int kStageWarp = kStageHalf + 512;
 
-__device__ __forceinline__ void bulk_add_u64x4(unsigned long long* gdst, unsigned long long* slot,
-                                               long long a0, long long a1, long long a2, long long e) {
-  asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-  reinterpret_cast<ulonglong2*>(slot)[0] = make_ulonglong2((unsigned long long)a0, (unsigned long long)a1);
-  reinterpret_cast<ulonglong2*>(slot)[1] = make_ulonglong2((unsigned long long)a2, (unsigned long long)e);
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(slot);
-  asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.u64 [%0], [%1], 32;"
-               :: "l"(gdst), "r"(sa) : "memory");
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-
-// wait for every bulk operation this thread issued (reads of shared memory
-// and the reductions in global memory)
-__device__ __forceinline__ void bulk_wait_all() {
-  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
+// with a single deposited value per crossing (pure H, isothermal) the record
+// has one nonzero: each lane then sends its own
+template <bool HE, bool HEAT>
 struct GlobalCells {
+  static constexpr bool kWarp = true;
   const float4* abs;
   unsigned long long* dep;
   int64_t coff;
   int nx, ny;
-  unsigned long long* stage;     // this thread's two 32-byte slots (shared), or nullptr
-  mutable int slot;
+  unsigned char* stage;          // this warp's staging area (shared)
   __device__ __forceinline__ int64_t index(int ix, int iy, int iz) const {
     return coff + (ix + nx * (iy + ny * iz));
   }
-  __device__ __forceinline__ float4 load(int64_t c, int, int, int) const { return __ldg(abs + c); }
-  __device__ __forceinline__ void add(int64_t c, long long a0, long long a1, long long a2, long long e) const {
-    unsigned long long* dp = dep + 4 * c;
-    if (stage) {
-      bulk_add_u64x4(dp, stage + 4 * slot, a0, a1, a2, e);
-      slot ^= 1;
+  __device__ __forceinline__ float4 load(int64_t c) const { return __ldg(abs + c); }
+  // called by the whole warp; has: this lane has a record for cell c
+  __device__ __forceinline__ void add(bool has, int64_t c, long long a0, long long a1, long long a2,
+                                      long long e) const {
+    if (!HE && !HEAT) {
+      if (has) atomicAdd(dep + 4 * c, (unsigned long long)a0);
       return;
     }
-    if (a0) atomicAdd(dp + 0, (unsigned long long)a0);
-    if (a1) atomicAdd(dp + 1, (unsigned long long)a1);
-    if (a2) atomicAdd(dp + 2, (unsigned long long)a2);
-    if (e) atomicAdd(dp + 3, (unsigned long long)e);
+    const unsigned mask = __ballot_sync(0xFFFFFFFFu, has);
+    if (mask == 0u) return;
+    const unsigned lane = threadIdx.x & 31;
+    if (has) {
+      *reinterpret_cast<ulonglong2*>(stage + 16 * lane) = make_ulonglong2((unsigned long long)a0, (unsigned long long)a1);
+      *reinterpret_cast<ulonglong2*>(stage + kStageHalf + 16 * lane) =
+          make_ulonglong2((unsigned long long)a2, (unsigned long long)e);
+    }
+    __syncwarp();
+    const unsigned k = lane & 3u, r0 = lane >> 2;
+    const unsigned char* src = stage + (k >> 1) * kStageHalf + 8 * (k & 1u) + 16 * r0;
+    unsigned long long* dk = dep + k;
+    // cells of all boxes together are below 2^32 (their state alone is 84 bytes a cell)
+    const unsigned c32 = (unsigned)c;
+#pragma unroll
+    for (unsigned q = 0; q < 4; ++q) {
+      const unsigned rc = __shfl_sync(0xFFFFFFFFu, c32, 8 * q + r0);
+      if ((mask >> (8 * q + r0)) & 1u) {
+        const unsigned long long v = *reinterpret_cast<const unsigned long long*>(src + 128 * q);
+        if (v) atomicAdd(dk + 4 * (size_t)rc, v);
+      }
+    }
+    __syncwarp();                // the next crossing's records overwrite the staging area
   }
 };
 
@@ -494,14 +504,17 @@ struct GlobalCells {
 // one array of 4096 per species (so that lanes at different cells spread
 // over the banks), and go to the grid once per work item
 struct TileCells {
+  static constexpr bool kWarp = false;
   const float4* sabs;              // shared, [16][16][16]
   unsigned long long* sdep;        // shared, [4][16][16][16]
   int x0, y0, z0;
   __device__ __forceinline__ int64_t index(int ix, int iy, int iz) const {
     return (ix - x0) + 16 * ((iy - y0) + 16 * (iz - z0));
   }
-  __device__ __forceinline__ float4 load(int64_t c, int, int, int) const { return sabs[c]; }
-  __device__ __forceinline__ void add(int64_t c, long long a0, long long a1, long long a2, long long e) const {
+  __device__ __forceinline__ float4 load(int64_t c) const { return sabs[c]; }
+  __device__ __forceinline__ void add(bool has, int64_t c, long long a0, long long a1, long long a2,
+                                      long long e) const {
+    if (!has) return;
     if (a0) atomicAdd(sdep + c, (unsigned long long)a0);
     if (a1) atomicAdd(sdep + 4096 + c, (unsigned long long)a1);
     if (a2) atomicAdd(sdep + 8192 + c, (unsigned long long)a2);
@@ -520,13 +533,17 @@ struct TileCells {
 // (ESCAPED) once the path trem (cells, the rest of c dt) is used up, the
 // last segment cut there (Sec. 2 periodic boxes).  The photons the walk
 // absorbed are counted once at its end, as the drop of the packet's content.
+// run: the lane has a packet.  With Cells::kWarp the whole warp walks
+// together (every lane calls, and lanes whose packet is done wait for the
+// last) because the warp sends its deposits together.
 template <int NBT, bool HE, bool HEAT, bool TILE, bool PER, class Cells>
-__device__ __forceinline__ int walk_steps(int& ix, int& iy, int& iz, float& tMx, float& tMy, float& tMz,
+__device__ __forceinline__ int walk_steps(const bool run, int& ix, int& iy, int& iz, float& tMx, float& tMy, float& tMz,
                                     const float dx, const float dy, const float dz, Content<NBT>& N,
                                     const BoxMeta* M, const Cells& cells, const BinTables& t,
                                     const int nb, const int max_iter, Tally& tl, int tx0 = 0,
                                     int ty0 = 0, int tz0 = 0, int ex = 0, int ey = 0, int ez = 0,
                                     float* trem = nullptr) {
+  if (max_iter <= 0) return ALIVE;
   const int nx = M->nx, ny = M->ny, nz = M->nz;
   const bool per = PER && M->periodic;
   const float tDx = dx != 0.f ? 1.0f / fabsf(dx) : INFINITY;
@@ -535,7 +552,6 @@ __device__ __forceinline__ int walk_steps(int& ix, int& iy, int& iz, float& tMx,
   const int sx = dx > 0.f ? 1 : -1, sy = dy > 0.f ? 1 : -1, sz = dz > 0.f ? 1 : -1;
   const float dl = M->dlf;
   const bool heat_box = HEAT && !M->isothermal;
-  if (max_iter <= 0) return ALIVE;
   unsigned left = 0;
 #pragma unroll
   for (int j = 0; j < (NBT > 0 ? NBT : CRASH_MAX_BINS); ++j)
@@ -543,93 +559,99 @@ __device__ __forceinline__ int walk_steps(int& ix, int& iy, int& iz, float& tMx,
   // current segment
   float seg = fminf(tMx, fminf(tMy, tMz));
   int ax = (tMx <= tMy && tMx <= tMz) ? 0 : (tMy <= tMz ? 1 : 2);
-  int64_t cell = cells.index(ix, iy, iz);
-  float4 ab = cells.load(cell, ix, iy, iz);
+  int64_t cell = 0;
+  float4 ab = make_float4(0.f, 0.f, 0.f, 0.f);
+  bool go = run;
+  int status = ALIVE;
+  if (go) {
+    cell = cells.index(ix, iy, iz);
+    ab = cells.load(cell);
+  }
   for (int it = 1;; ++it) {
-    // step the walk into the next cell and request its absorbers
-    const bool bx = ax == 0, by = ax == 1, bz = ax == 2;
-    tMx = bx ? tDx : tMx - seg;
-    tMy = by ? tDy : tMy - seg;
-    tMz = bz ? tDz : tMz - seg;
-    ix += bx ? sx : 0;
-    iy += by ? sy : 0;
-    iz += bz ? sz : 0;
-    if (PER && per) {
-      ix = ix < 0 ? nx - 1 : (ix >= nx ? 0 : ix);
-      iy = iy < 0 ? ny - 1 : (iy >= ny ? 0 : iy);
-      iz = iz < 0 ? nz - 1 : (iz >= nz ? 0 : iz);
+    if (Cells::kWarp ? !__any_sync(0xFFFFFFFFu, go) : !go) return status;
+    const int64_t at = cell;
+    bool has = false;
+    long long dHI = 0, dHeI = 0, dHeII = 0, dE = 0;
+    if (go) {
+      // step the walk into the next cell and request its absorbers
+      const bool bx = ax == 0, by = ax == 1, bz = ax == 2;
+      tMx = bx ? tDx : tMx - seg;
+      tMy = by ? tDy : tMy - seg;
+      tMz = bz ? tDz : tMz - seg;
+      ix += bx ? sx : 0;
+      iy += by ? sy : 0;
+      iz += bz ? sz : 0;
+      if (PER && per) {
+        ix = ix < 0 ? nx - 1 : (ix >= nx ? 0 : ix);
+        iy = iy < 0 ? ny - 1 : (iy >= ny ? 0 : iy);
+        iz = iz < 0 ? nz - 1 : (iz >= nz ? 0 : iz);
+      }
+      const bool out = ((unsigned)ix >= (unsigned)nx) | ((unsigned)iy >= (unsigned)ny) |
+                       ((unsigned)iz >= (unsigned)nz);
+      const bool leave = TILE ? (((unsigned)(ix - tx0) >= (unsigned)ex) | ((unsigned)(iy - ty0) >= (unsigned)ey) |
+                                 ((unsigned)(iz - tz0) >= (unsigned)ez))
+                              : out;
+      float seg_n = 0.f;
+      int ax_n = 0;
+      float4 ab_n = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (!leave) {
+        seg_n = fminf(tMx, fminf(tMy, tMz));
+        ax_n = (tMx <= tMy && tMx <= tMz) ? 0 : (tMy <= tMz ? 1 : 2);
+        cell = cells.index(ix, iy, iz);
+        ab_n = cells.load(cell);
+      }
+      // periodic: the path left to the light-travel distance cuts the segment
+      bool stop = false;
+      if (PER && per) {
+        stop = seg >= *trem;
+        if (stop) seg = *trem;
+        *trem -= seg;
+      }
+      if (PER && stop) { go = false; status = ESCAPED; }
+      else if (out) { go = false; status = ESCAPED; }
+      else if ((TILE && leave) || it >= max_iter) go = false;
+      // attenuate and deposit in the current cell
+      if (seg > 0.f) {
+        has = cell_attenuate<NBT, HE, HEAT>(seg, dl, ab, N, nb, t, dHI, dHeI, dHeII, dE, left) != 0;
+        tl.crossings += 1;
+        if (left == 0) { go = false; status = ABSORBED; }
+        if (!heat_box) dE = 0;
+      }
+      seg = seg_n;
+      ax = ax_n;
+      ab = ab_n;
     }
-    const bool out = ((unsigned)ix >= (unsigned)nx) | ((unsigned)iy >= (unsigned)ny) |
-                     ((unsigned)iz >= (unsigned)nz);
-    const bool leave = TILE ? (((unsigned)(ix - tx0) >= (unsigned)ex) | ((unsigned)(iy - ty0) >= (unsigned)ey) |
-                               ((unsigned)(iz - tz0) >= (unsigned)ez))
-                            : out;
-    float seg_n = 0.f;
-    int ax_n = 0;
-    int64_t cell_n = cell;
-    float4 ab_n = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!leave) {
-      seg_n = fminf(tMx, fminf(tMy, tMz));
-      ax_n = (tMx <= tMy && tMx <= tMz) ? 0 : (tMy <= tMz ? 1 : 2);
-      cell_n = cells.index(ix, iy, iz);
-      ab_n = cells.load(cell_n, ix, iy, iz);
-    }
-    // periodic: the path left to the light-travel distance cuts the segment
-    bool stop = false;
-    if (PER && per) {
-      stop = seg >= *trem;
-      if (stop) seg = *trem;
-      *trem -= seg;
-    }
-    // attenuate and deposit in the current cell
-    if (seg > 0.f) {
-      long long dHI, dHeI, dHeII, dE;
-      const long long Atot = cell_attenuate<NBT, HE, HEAT>(seg, dl, ab, N, nb, t, dHI, dHeI, dHeII,
-                                                           dE, left);
-      if (Atot) cells.add(cell, dHI, dHeI, dHeII, heat_box ? dE : 0ll);
-      tl.crossings += 1;
-      if (left == 0) return ABSORBED;
-    }
-    if (PER && stop) return ESCAPED;
-    if (out) return ESCAPED;
-    if (TILE && leave) return ALIVE;
-    if (it >= max_iter) return ALIVE;
-    seg = seg_n;
-    ax = ax_n;
-    cell = cell_n;
-    ab = ab_n;
+    cells.add(has, at, dHI, dHeI, dHeII, dE);
   }
 }
 
 template <int NBT, bool HE, bool HEAT, bool TILE, bool PER, class Cells>
-__device__ __forceinline__ int walk(int& ix, int& iy, int& iz, float& tMx, float& tMy, float& tMz,
+__device__ __forceinline__ int walk(const bool run, int& ix, int& iy, int& iz, float& tMx, float& tMy, float& tMz,
                                     const float dx, const float dy, const float dz, Content<NBT>& N,
                                     const BoxMeta* M, const Cells& cells, const BinTables& t,
                                     const int nb, const int max_iter, Tally& tl, int tx0 = 0,
                                     int ty0 = 0, int tz0 = 0, int ex = 0, int ey = 0, int ez = 0,
                                     float* trem = nullptr) {
-  tl.absorbed += N.total(nb);
-  const int r = walk_steps<NBT, HE, HEAT, TILE, PER>(ix, iy, iz, tMx, tMy, tMz, dx, dy, dz, N, M, cells, t,
+  if (run) tl.absorbed += N.total(nb);
+  const int r = walk_steps<NBT, HE, HEAT, TILE, PER>(run, ix, iy, iz, tMx, tMy, tMz, dx, dy, dz, N, M, cells, t,
                                                      nb, max_iter, tl, tx0, ty0, tz0, ex, ey, ez, trem);
-  tl.absorbed -= N.total(nb);
+  if (run) tl.absorbed -= N.total(nb);
   return r;
 }
 
-// the walk over the grid in global memory
+// the walk over the grid in global memory (called by whole warps; run: this
+// lane has a packet, M is then its box and else any box)
 template <int NBT, bool HE, bool HEAT, bool PER = false>
-__device__ __forceinline__ int trace_mixed(int& ix, int& iy, int& iz, float& tMx, float& tMy,
+__device__ __forceinline__ int trace_mixed(const bool run, int& ix, int& iy, int& iz, float& tMx, float& tMy,
                                            float& tMz, const float dx, const float dy,
                                            const float dz, Content<NBT>& N, const BoxMeta* M,
                                            const StepArgs& a, const BinTables& t, const int nb,
                                            const int max_iter, Tally& tl, float* trem = nullptr) {
-  __shared__ __align__(16) unsigned long long stage[kStageThreads * 8];
-  const bool bulk = threadIdx.x < kStageThreads && ((uintptr_t)a.dep & 15u) == 0;
-  GlobalCells cells{reinterpret_cast<const float4*>(a.abs32), a.dep, M->cell_off, M->nx, M->ny,
-                    bulk ? stage + 8 * threadIdx.x : nullptr, 0};
-  const int r = walk<NBT, HE, HEAT, false, PER>(ix, iy, iz, tMx, tMy, tMz, dx, dy, dz, N, M, cells, t,
-                                                nb, max_iter, tl, 0, 0, 0, 0, 0, 0, trem);
-  if (bulk) bulk_wait_all();
-  return r;
+  __shared__ __align__(16) unsigned char stage[(HE || HEAT) ? kMaxWarps * kStageWarp : 16];
+  const GlobalCells<HE, HEAT> cells{reinterpret_cast<const float4*>(a.abs32), a.dep, M->cell_off, M->nx, M->ny,
+                                    stage + ((HE || HEAT) ? (threadIdx.x >> 5) * kStageWarp : 0)};
+  return walk<NBT, HE, HEAT, false, PER>(run, ix, iy, iz, tMx, tMy, tMz, dx, dy, dz, N, M, cells, t,
+                                         nb, max_iter, tl, 0, 0, 0, 0, 0, 0, trem);
 }
 
 // warp-aggregated append of surviving packets to the output queue
@@ -771,12 +793,14 @@ __device__ __forceinline__ void emit_range(const StepArgs& a, const BinTables& t
     bool alive = false;
     int ix = 0, iy = 0, iz = 0;
     float tMx = 0.f, tMy = 0.f, tMz = 0.f, fx = 0.f, fy = 0.f, fz = 0.f;
-    Content<NBT> N;
-    N.e = 0;
+    Content<NBT> N{};
+    const BoxMeta* M = a.boxes;
+    float trem = 0.f;
+    bool run = false;
     if (i < n) {
       const int64_t gid = g0 + i;
       b = box_of_packet(a.boxes, a.n_boxes, gid);
-      const BoxMeta* M = a.boxes + b;
+      M = a.boxes + b;
       const int64_t local = gid - M->pkt_off;
       const uint32_t W = M->win_hi - M->win_lo;
       const int s_local = (int)(local / W);
@@ -807,14 +831,17 @@ __device__ __forceinline__ void emit_range(const StepArgs& a, const BinTables& t
         tMx = fx > 0.f ? ((float)(ix + 1) - px) / fx : (fx < 0.f ? ((float)ix - px) / fx : INFINITY);
         tMy = fy > 0.f ? ((float)(iy + 1) - py) / fy : (fy < 0.f ? ((float)iy - py) / fy : INFINITY);
         tMz = fz > 0.f ? ((float)(iz + 1) - pz) / fz : (fz < 0.f ? ((float)iz - pz) / fz : INFINITY);
-        float trem = PER ? M->path_cells32 : 0.f;
-        const int r = trace_mixed<NBT, HE, HEAT, PER>(ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, a, t,
-                                                      nb, S, tl, &trem);
-        if (r == ESCAPED) tl.escaped += N.total(nb);
-        alive = (r == ALIVE);
-        // traced to the end (no queue to keep it): a packet still alive hit the DDA bound
-        if (alive && S >= max_steps_all) atomicOr(a.err, ERR_DDA_LIMIT);
+        trem = PER ? M->path_cells32 : 0.f;
+        run = true;
       }
+    }
+    const int r = trace_mixed<NBT, HE, HEAT, PER>(run, ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, a, t, nb, S, tl,
+                                                  &trem);
+    if (run) {
+      if (r == ESCAPED) tl.escaped += N.total(nb);
+      alive = (r == ALIVE);
+      // traced to the end (no queue to keep it): a packet still alive hit the DDA bound
+      if (alive && S >= max_steps_all) atomicOr(a.err, ERR_DDA_LIMIT);
     }
     if (S < max_steps_all)   // a wavefront launch: keep the survivors
       write_survivor<NBT>(a, w, alive, ix, iy, iz, b, tMx, tMy, tMz, fx, fy, fz, N, nb);
@@ -842,13 +869,17 @@ __global__ void __launch_bounds__(256, 3) k_rec_mixed(StepArgs a, BinTables t) {
     const int64_t e = base + threadIdx.x;
     Tally tl{0, 0, 0, 0u, 0u};
     int b = -1;
+    bool run = false;
+    const BoxMeta* M = a.boxes;
+    Content<NBT> N{};
+    int ix = 0, iy = 0, iz = 0;
+    float tMx = 0.f, tMy = 0.f, tMz = 0.f, fx = 0.f, fy = 0.f, fz = 0.f, trem = 0.f;
     if (e < n) {
       const long long* L = a.rec_list + 4 * e;
       const int64_t g = L[0];
       b = box_of_cell(a.boxes, a.n_boxes, g);
-      const BoxMeta* M = a.boxes + b;
+      M = a.boxes + b;
       const int64_t cell = g - M->cell_off;
-      float fx, fy, fz;
       if (!iso_direction_f32(M->seed, step, rec_src_id(cell), (uint32_t)cell, fx, fy, fz)) {
         atomicOr(a.err, ERR_DIRECTION);
       } else {
@@ -858,7 +889,6 @@ __global__ void __launch_bounds__(256, 3) k_rec_mixed(StepArgs a, BinTables t) {
           if (a.rec_bin[s] >= 0) q[a.rec_bin[s]] += (unsigned long long)L[1 + s];
         unsigned long long qmax = 0;
         for (int j = 0; j < nb; ++j) qmax = q[j] > qmax ? q[j] : qmax;
-        Content<NBT> N;
         const int bits = qmax ? 64 - __clzll((long long)qmax) : 0;
         N.e = bits > 32 ? bits - 32 : 0;
         for (int j = 0; j < nb; ++j) N.m[j] = (unsigned)(q[j] >> N.e);
@@ -866,19 +896,23 @@ __global__ void __launch_bounds__(256, 3) k_rec_mixed(StepArgs a, BinTables t) {
         tl.packets += 1;
         double ox, oy, oz;
         rec_offsets(M->seed, step, cell, ox, oy, oz);
-        int ix = (int)(cell % M->nx), iy = (int)((cell / M->nx) % M->ny);
-        int iz = (int)(cell / ((int64_t)M->nx * M->ny));
+        ix = (int)(cell % M->nx);
+        iy = (int)((cell / M->nx) % M->ny);
+        iz = (int)(cell / ((int64_t)M->nx * M->ny));
         const float px = (float)((double)ix + ox), py = (float)((double)iy + oy);
         const float pz = (float)((double)iz + oz);
-        float tMx = fx > 0.f ? ((float)(ix + 1) - px) / fx : (fx < 0.f ? ((float)ix - px) / fx : INFINITY);
-        float tMy = fy > 0.f ? ((float)(iy + 1) - py) / fy : (fy < 0.f ? ((float)iy - py) / fy : INFINITY);
-        float tMz = fz > 0.f ? ((float)(iz + 1) - pz) / fz : (fz < 0.f ? ((float)iz - pz) / fz : INFINITY);
-        float trem = PER ? M->path_cells32 : 0.f;
-        const int r = trace_mixed<NBT, HE, HEAT, PER>(ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, a, t,
-                                                      nb, M->max_iter, tl, &trem);
-        if (r == ESCAPED) tl.escaped += N.total(nb);
-        else if (r == ALIVE) atomicOr(a.err, ERR_DDA_LIMIT);
+        tMx = fx > 0.f ? ((float)(ix + 1) - px) / fx : (fx < 0.f ? ((float)ix - px) / fx : INFINITY);
+        tMy = fy > 0.f ? ((float)(iy + 1) - py) / fy : (fy < 0.f ? ((float)iy - py) / fy : INFINITY);
+        tMz = fz > 0.f ? ((float)(iz + 1) - pz) / fz : (fz < 0.f ? ((float)iz - pz) / fz : INFINITY);
+        trem = PER ? M->path_cells32 : 0.f;
+        run = true;
       }
+    }
+    const int r = trace_mixed<NBT, HE, HEAT, PER>(run, ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, a, t, nb,
+                                                  a.max_iter_step, tl, &trem);
+    if (run) {
+      if (r == ESCAPED) tl.escaped += N.total(nb);
+      else if (r == ALIVE) atomicOr(a.err, ERR_DDA_LIMIT);
     }
     flush_warp(a, b, tl);
   }
@@ -917,9 +951,10 @@ __device__ __forceinline__ void pass_range(const StepArgs& a, const BinTables& t
     if (j < n) {
       const int64_t i = w.perm ? (int64_t)__ldcg(w.perm + j) : j;
       load_record<NBT>(w.rec_in, w.rs, i, ix, iy, iz, b, tMx, tMy, tMz, fx, fy, fz, N, nb);
-      const BoxMeta* M = a.boxes + b;
-      const int r = trace_mixed<NBT, HE, HEAT>(ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, a, t,
-                                               nb, S, tl);
+    }
+    const BoxMeta* M = a.boxes + (b < 0 ? 0 : b);
+    const int r = trace_mixed<NBT, HE, HEAT>(b >= 0, ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, a, t, nb, S, tl);
+    if (b >= 0) {
       if (r == ESCAPED) tl.escaped += N.total(nb);
       alive = (r == ALIVE);
     }
@@ -955,9 +990,10 @@ __device__ __forceinline__ void pass_range_q(const StepArgs& a, const BinTables&
     if (j < n) {
       const int64_t i = read_sorted ? (int64_t)__ldcg(wf.perm + j) : j;
       load_record<NBT>(wf.rec[CUR], wf.rs, i, ix, iy, iz, b, tMx, tMy, tMz, fx, fy, fz, N, nb);
-      const BoxMeta* M = a.boxes + b;
-      const int r = trace_mixed<NBT, HE, HEAT>(ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, a, t,
-                                               nb, S, tl);
+    }
+    const BoxMeta* M = a.boxes + (b < 0 ? 0 : b);
+    const int r = trace_mixed<NBT, HE, HEAT>(b >= 0, ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, a, t, nb, S, tl);
+    if (b >= 0) {
       if (r == ESCAPED) tl.escaped += N.total(nb);
       alive = (r == ALIVE);
     }
@@ -1153,7 +1189,7 @@ __global__ void __launch_bounds__(kTileBlock, 1) k_tile_pass(StepArgs a, BinTabl
       if (j < hi) {
         load_record<NBT>(w.rec_in, w.rs, (long long)w.perm[j], ix, iy, iz, pb, tMx, tMy, tMz, fx, fy, fz,
                          N, nb);
-        const int r = walk<NBT, HE, HEAT, true, false>(ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, cells,
+        const int r = walk<NBT, HE, HEAT, true, false>(true, ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, cells,
                                                        t, nb, 64, tl, x0, y0, z0, ex, ey, ez);
         if (r == ESCAPED) tl.escaped += N.total(nb);
         alive = (r == ALIVE);
