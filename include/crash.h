@@ -134,7 +134,14 @@ typedef struct {
   int seg_per_iter;          /* mixed form: crossings per packet per wavefront pass (0 = tuned) */
   int resort_interval;       /* mixed form: wavefront passes between Morton re-sorts (0 = tuned,
                                 <0 = never) */
-  int wavefront;             /* mixed form: 1 = packet-queue wavefront, 0 = one thread per packet */
+  int wavefront;             /* mixed form: 0 = one thread per packet in emission order.  1 (default)
+                                = the library orders the packets: with seg_per_iter,
+                                resort_interval, pass_limit and tile all 0 it chooses by the
+                                step's sizes (emission order for few packets, bundles sorted by
+                                source and direction and traced to the end, or wavefront passes
+                                over a packet queue for large grids with many sources); any of
+                                them nonzero asks for wavefront passes.  Results do not depend
+                                on it. */
   int use_graph;             /* 1: capture each step in a CUDA graph and replay it */
   int timing;                /* 1: record CUDA events around the transport launches */
   int reg_cap;               /* mixed form: 1 = transport kernels capped at 64 registers
@@ -151,14 +158,15 @@ typedef struct {
                                 0 = Morton (Z) curve, 1 = Hilbert curve; tile passes
                                 (tile = 1) always key by Morton tiles.  Results do not
                                 depend on it (only the order packets are traced in). */
-  int chunk_packets;         /* mixed form: packets per wavefront chunk (0 = 2^28); a step
-                                with more packets runs chunk after chunk through one queue.
-                                Results do not depend on it. */
-  int persistent;            /* mixed form, wavefront without tiles: 1 = the whole transport
-                                of a step in one cooperative launch whose blocks stay
-                                resident and meet at grid barriers between passes and
-                                re-sort phases (default); 0 = one launch per pass and per
-                                re-sort phase.  Every barrier wait is bounded (30 s), after
+  int chunk_packets;         /* mixed form: packets per bundle or wavefront chunk (0 = 2^28); a
+                                step with more packets runs chunk after chunk through one
+                                workspace.  Results do not depend on it. */
+  int persistent;            /* mixed form, wavefront passes asked for (see wavefront) without
+                                tiles: 1 = the whole transport of a step in one cooperative
+                                launch whose blocks stay resident and meet at grid barriers
+                                between passes and re-sort phases (default); 0 = one launch per
+                                pass and per re-sort phase, as in the passes the library
+                                chooses by itself.  Every barrier wait is bounded (30 s), after
                                 which the step reports CRASH_ERR_TIMEOUT.  Results do not
                                 depend on it. */
 } crash_run_opts;
@@ -249,7 +257,8 @@ int64_t crash_launch_count(crash_ctx* ctx);
    (opts.persistent); the state, the diffuse field's counts and the step
    index are restored afterwards.  Stores the fastest in the context's
    options (persistent included) and returns the chosen values (outputs may
-   be NULL). */
+   be NULL).  The form the library chooses by itself (seg_per_iter and
+   resort_interval 0) is one of the trials. */
 crash_status crash_autotune(crash_ctx* ctx, double dt_s, const uint64_t* packets_per_box,
                             int* block_size, int* seg_per_iter, int* resort_interval,
                             int* reg_cap, int* tile, int* sort_curve);
@@ -290,9 +299,9 @@ const char* crash_last_error(crash_ctx* ctx);   /* NULL ctx: last creation error
    are handed).  It runs the mixed-form transport of one grid for one step
    (emission, cell walk, attenuation, int64 deposition; no chemistry, no
    re-sort) exactly as crash_step does for a context with the same grid,
-   sources and options, and allocates nothing: its scratch (packet queue of
-   65536 packets per pass buffer, per-source tables for at most
-   CRASH_NOALLOC_MAX_SOURCES sources, counters; about 21 MB) is a static
+   sources and options, and allocates nothing: its scratch (sort buffers of
+   2^20 packets, or a packet queue of 65536 packets per pass buffer, per-source
+   tables for at most CRASH_NOALLOC_MAX_SOURCES sources, counters; about 21 MB) is a static
    device array that every GPU loading the library holds until the process
    exits.
      grid: host struct; nx, ny, nz, box_cm, he_over_h, isothermal, caseB and
@@ -304,7 +313,8 @@ const char* crash_last_error(crash_ctx* ctx);   /* NULL ctx: last creation error
      dt_s, step_index, packets_per_step: as in crash_step (step_index is the
        Philox step word); packets_per_step <= CRASH_NOALLOC_MAX_PACKETS
        (larger steps: CRASH_ERR_OVERFLOW); seg_per_pass: cells per wavefront
-       pass (0 = 32).
+       pass (0: no passes, packets sorted by source and direction and traced
+       to the end).
      absorbers_dev: device float[nx*ny*nz][4] = n_HI, n_HeI, n_HeII, 0 (cm^-3),
        16-byte aligned (CRASH_ERR_ARG otherwise).
      deposits_dev: device uint64[nx*ny*nz][4] (HI, HeI, HeII, heat), 8-byte
@@ -323,7 +333,7 @@ const char* crash_last_error(crash_ctx* ctx);   /* NULL ctx: last creation error
    arguments (nothing is launched), CRASH_ERR_CUDA, CRASH_ERR_TIMEOUT for a
    device-side bound; crash_noalloc_last_error() gives the message. */
 #define CRASH_NOALLOC_MAX_SOURCES 1024
-#define CRASH_NOALLOC_MAX_PACKETS (1ull << 30)   /* 16384 queue chunks of 65536 packets */
+#define CRASH_NOALLOC_MAX_PACKETS (1ull << 30)   /* 1024 chunks of 2^20 packets, 16384 of 65536 in passes */
 crash_status crash_transport_noalloc(const crash_grid_desc* grid, int n_src, const double* pos_cells,
                                      const double* ndot, int n_bins, const double* bin_eV,
                                      const double* bin_frac, double dt_s, uint64_t step_index,

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <algorithm>
@@ -96,9 +97,19 @@ struct crash_ctx {
   int64_t n_keys = 0;            // wavefront re-sort keys over all boxes
   int64_t n_tile_keys = 0;       // tile-pass keys over all boxes
   int max_tiles = 0;             // bound on the tiles one packet crosses
-  int wf_mode = -1;              // wavefront option the workspace was sized for
   size_t bytes = 0;              // device bytes allocated by the context
 };
+
+// L2 cache of the current device
+static int64_t l2_bytes() {
+  static const int64_t n = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    return cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, dev) == cudaSuccess && v > 0 ? (int64_t)v
+                                                                                          : (int64_t)126 << 20;
+  }();
+  return n;
+}
 
 // optional cap on the device memory a context may allocate (bytes; 0 = none)
 static size_t memory_cap() {
@@ -280,17 +291,23 @@ extern "C" crash_status crash_init_batch(int n_boxes, const crash_grid_desc* des
     c->any_heat |= !d.isothermal;
   }
   c->n_cells = off;
-  // wavefront sort keys: per box, Morton order of 8^3-cell buckets times 8 octants
+  // wavefront sort keys: per box, Morton order of 8^3-cell buckets times 64
+  // direction cells, or 16, or the 8 octants, as the scan has room for
   int64_t keys = 0;
-  for (int i = 0; i < n_boxes; ++i) {
-    BoxMeta& m = c->meta[i];
-    int cmax = std::max(std::max((m.nx + 7) / 8, (m.ny + 7) / 8), (m.nz + 7) / 8);
-    int bits = 0;
-    while ((1 << bits) < cmax) ++bits;
-    m.bucket_bits = bits;
-    m.bucket_off = keys;
-    keys += (int64_t)8 << (3 * bits);
-    c->max_iter = std::max(c->max_iter, m.max_iter);
+  for (int dir_bits : {3, 2, 0}) {
+    keys = 0;
+    for (int i = 0; i < n_boxes; ++i) {
+      BoxMeta& m = c->meta[i];
+      int cmax = std::max(std::max((m.nx + 7) / 8, (m.ny + 7) / 8), (m.nz + 7) / 8);
+      int bits = 0;
+      while ((1 << bits) < cmax) ++bits;
+      m.bucket_bits = bits;
+      m.bucket_off = keys;
+      m.dir_bits = dir_bits;
+      keys += (int64_t)(dir_bits ? 1 << (2 * dir_bits) : 8) << (3 * bits);
+      c->max_iter = std::max(c->max_iter, m.max_iter);
+    }
+    if (keys <= (int64_t)4096 * 1024) break;
   }
   c->n_keys = keys;
   // tile-pass keys: 16^3-cell tiles times 8 octants (fewer than the 8^3 keys)
@@ -611,6 +628,7 @@ static StepArgs make_args(crash_ctx* c, double dt, int64_t total) {
   StepArgs a;
   memset(&a, 0, sizeof a);
   a.boxes = c->d_meta;
+  a.boxes_host = c->meta.data();
   a.n_boxes = c->n_boxes;
   a.step_dev = c->step_dev;
   a.dt = dt;
@@ -716,6 +734,35 @@ static crash_status enqueue_step(crash_ctx* c, const StepArgs& a, bool timing, i
   return CRASH_OK;
 }
 
+// a pass length, a re-sort interval, a pass limit or tiles ask for passes
+static bool passes_asked(const crash_run_opts& o) {
+  return o.tile || o.seg_per_iter > 0 || o.resort_interval != 0 || o.pass_limit > 0;
+}
+
+// Form of the mixed transport of a step of `total` packets (the results do
+// not depend on it).
+static int transport_form(const crash_ctx* c, int64_t total) {
+  const crash_run_opts& o = c->opts;
+  if (!o.wavefront) return FORM_DIRECT;
+  // (periodic boxes have no passes: their packets' path budget is not in a record)
+  if (!c->any_periodic && passes_asked(o)) return FORM_PASSES;
+  if (total <= resident_packets()) return FORM_DIRECT;
+  if (c->n_src_total > kMaxBundleKeys) return c->any_periodic ? FORM_DIRECT : FORM_PASSES;
+  if (c->any_periodic) return FORM_BUNDLE;
+  // A bundle's 32 packets spread to about w cells at half the grid's width,
+  // w^2 = (n / 2)^2 4 pi 32 / (packets per source).  Where absorbers and
+  // deposits (48 bytes a cell) do not fit L2, wide bundles miss it, and passes
+  // in spatial order win if they have packets enough to fill their buckets:
+  // 20e6 packets, thin, ms for bundles / passes: 192^3 2000 sources (w = 19)
+  // 54 / 40, 1000 sources of 60e6 (8) 118 / 117, 300 (7) 39 / 41, 1 source 35
+  // / 45; 256^3 2000 sources (26) 78 / 52, 100 (6) 45 / 51; 1e6 packets, 1000
+  // sources (81) 5.7 / 6.9.  128^3 fits L2: 2000 sources (13) 25.5 / 25.6.
+  int64_t most = 0;
+  for (const BoxMeta& m : c->meta) most = std::max(most, m.ncell);
+  const double n2 = pow((double)most, 2.0 / 3.0), per_source = (double)total / (double)c->n_src_total;
+  if (48 * c->n_cells > l2_bytes() && per_source < 1.25 * n2 && total > c->n_cells / 4) return FORM_PASSES;
+  return FORM_BUNDLE;
+}
 extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t* P) {
   if (!c) return CRASH_ERR_ARG;
   if (!(dt > 0) || !isfinite(dt)) return set_err(c, CRASH_ERR_ARG, "dt must be positive");
@@ -761,15 +808,30 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
   }
   CK(cudaMemcpyAsync(c->d_meta, c->meta.data(), sizeof(BoxMeta) * c->n_boxes,
                      cudaMemcpyHostToDevice, c->stream));
+  int form = FORM_DIRECT;
+  bool per_launch = false;
   if (c->precision == CRASH_MIXED) {
-    // packet queue: sized to the step (at most 2^28 packets per chunk, 38 GB
-    // with 8 bins); none when every packet is traced to the end by its own
-    // thread.  Larger chunks put more packets in each sort bucket of a pass,
-    // so more crossings of a cell fall close together in time and its
-    // deposit record is reused in L2.
+    // workspace: the packet queue (two record buffers) or the sort buffers
+    // of the step's form, sized to the step (at most 2^28 packets per chunk:
+    // 38 GB of queue with 8 bins, 3.2 GB of sort buffers); none when every
+    // packet is traced to the end in emission order.
+    form = transport_form(c, total);
+    per_launch = form == FORM_PASSES && !passes_asked(c->opts);
     const int64_t chunk = c->opts.chunk_packets > 0 ? (int64_t)c->opts.chunk_packets : (int64_t)1 << 28;
-    const int64_t want = (c->opts.wavefront && !c->any_periodic) ? std::min<int64_t>(total, chunk) : 0;
-    if (c->wf && (c->wf_mode != c->opts.wavefront || wavefront_capacity(c->wf) < want)) {
+    WFSize want;
+    if (form == FORM_PASSES) {
+      want.queue = std::min<int64_t>(total, chunk);
+      want.n_keys = c->n_keys;
+    } else if (form == FORM_BUNDLE) {
+      want.bundle = std::min<int64_t>(total, chunk);
+      want.bundle_keys = std::max<int64_t>(c->n_src_total, std::min<int64_t>(kMaxBundleKeys, want.bundle / 2));
+    }
+    const WFSize have = wavefront_size(c->wf);
+    if (c->wf && (have.queue < want.queue || have.bundle < want.bundle || have.bundle_keys < want.bundle_keys)) {
+      want.queue = std::max(want.queue, have.queue);       // steps of both forms may alternate
+      want.n_keys = want.queue > 0 ? c->n_keys : 0;
+      want.bundle = std::max(want.bundle, have.bundle);
+      want.bundle_keys = std::max(want.bundle_keys, have.bundle_keys);
       CK(cudaStreamSynchronize(c->stream));
       wavefront_destroy(c->wf);
       c->wf = nullptr;
@@ -777,17 +839,19 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
     }
     if (!c->wf) {
       const size_t cap = memory_cap();
-      const size_t need = (size_t)want * (size_t)(2 * (((32 + 4 * c->n_bins) + 15) / 16 * 16) + 12);
+      const size_t need = (size_t)want.queue * (size_t)(2 * (((32 + 4 * c->n_bins) + 15) / 16 * 16)) +
+                          12 * (size_t)std::max(want.queue, want.bundle) + 8 * (size_t)want.bundle_keys;
       if (cap && c->bytes + need > cap)
-        return set_err(c, CRASH_ERR_OOM, "device memory cap (CRASH_DEVICE_MEMORY_CAP) exceeded by the packet queue");
+        return set_err(c, CRASH_ERR_OOM, "device memory cap (CRASH_DEVICE_MEMORY_CAP) exceeded by the packet workspace");
       cudaError_t e = cudaSuccess;
-      c->wf = wavefront_create(want, c->n_keys, c->n_bins, &e);
-      if (!c->wf) return set_err(c, CRASH_ERR_OOM, std::string("wavefront workspace: ") + cudaGetErrorString(e));
-      c->wf_mode = c->opts.wavefront;
+      c->wf = wavefront_create(want, c->n_bins, &e);
+      if (!c->wf) return set_err(c, CRASH_ERR_OOM, std::string("packet workspace: ") + cudaGetErrorString(e));
     }
   }
   StepArgs a = make_args(c, dt, total);
   a.max_iter_step = step_max_iter;
+  a.form = form;
+  a.launch_per_pass = per_launch;
   const bool timing = c->opts.timing != 0;
   crash_status st;
   if (c->opts.use_graph && !timing) {
@@ -1058,14 +1122,20 @@ extern "C" crash_status crash_autotune(crash_ctx* c, double dt, const uint64_t* 
     for (int bs : blocks)
       for (int sg : segs)
         for (int rs : resorts) trials.push_back({bs, sg, rs, cap, 0});
-  if (c->precision == CRASH_MIXED) trials.push_back({256, 0, 1, 0, 1});
+  if (c->precision == CRASH_MIXED) {
+    trials.push_back({256, 0, 1, 0, 1});
+    trials.push_back({256, 0, 0, 0, 0});      // the form the library chooses by itself
+  }
   // the grid of trials runs one launch per pass; the fastest configuration is
   // then tried once more with Hilbert-ordered bucket keys, and the fastest of
   // those once more as one persistent launch per step
   const int n_grid = (int)trials.size();
   for (int ti = 0; ti < n_grid + 2; ++ti) {
     const bool curve_trial = ti == n_grid, pers_trial = ti == n_grid + 1;
-    if ((curve_trial || pers_trial) && (c->precision != CRASH_MIXED || best.tile || best_ms >= 1e300)) break;
+    // (tiles, and the library's own form, have neither)
+    if ((curve_trial || pers_trial) &&
+        (c->precision != CRASH_MIXED || best.tile || best_ms >= 1e300 || !passes_asked(best)))
+      break;
     const Trial tr = ti >= n_grid ? Trial{best.block_size, best.seg_per_iter, best.resort_interval,
                                           best.reg_cap, best.tile}
                                   : trials[ti];

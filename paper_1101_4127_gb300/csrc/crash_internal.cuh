@@ -41,9 +41,11 @@ struct BoxMeta {
   int64_t pkt_off;         // first global packet slot of this box in the launch
   int64_t pkt_count;       // n_src * (win_hi - win_lo)
   // wavefront re-sort: keys of this box start at bucket_off; a key is
-  // morton(ix >> 3, iy >> 3, iz >> 3) (bucket_bits bits per axis) * 8 + octant
+  // morton(ix >> 3, iy >> 3, iz >> 3) (bucket_bits bits per axis), then one of
+  // 4^dir_bits direction cells (dir_bits = 0: one of 8 octants)
   int64_t bucket_off;
   int bucket_bits;
+  int dir_bits;
   // tile passes: keys of this box start at tile_off; a key is
   // morton(ix >> 4, iy >> 4, iz >> 4) (tile_bits bits per axis) * 8 + octant
   int64_t tile_off;
@@ -73,8 +75,18 @@ struct BinTables {
   float sw32[3][CRASH_MAX_BINS];     // sigma32 * wheat32 (FP32 product): heating weight per unit t_s
 };
 
+// Forms of the mixed transport (chosen per step by transport_form):
+//   FORM_DIRECT  one thread per packet, in emission order, traced to the end
+//   FORM_BUNDLE  the same, the packets sorted by source and direction first
+//   FORM_PASSES  the packet queue: passes of a few cells with spatial re-sorts,
+//                or tile passes
+enum { FORM_DIRECT = 0, FORM_BUNDLE = 1, FORM_PASSES = 2 };
+
 struct StepArgs {
   const BoxMeta* boxes;
+  const BoxMeta* boxes_host;      // the same table in host memory (launch code only)
+  int form;                       // mixed form: FORM_*
+  int launch_per_pass;            // passes chosen by the library: one launch each, 64 registers
   int n_boxes;
   unsigned long long* step_dev;   // step index (Philox counter word), advanced on the device
   double dt;
@@ -143,15 +155,29 @@ typedef std::vector<std::pair<cudaEvent_t, cudaEvent_t>> EventPairs;
 int launch_trace_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o,
                        void* wf_state, int max_iter, cudaStream_t s, EventPairs* ev, int* ev_used);
 
-// Mixed-form wavefront over caller-provided record buffers (no allocation,
-// no re-sort): rec0/rec1 hold cap records each, count holds 4 counters.
-int launch_trace_mixed_external(const StepArgs& a, const BinTables& t, const crash_run_opts& o,
-                                char* rec0, char* rec1, unsigned* count, int64_t cap, int max_iter,
-                                cudaStream_t s);
+// Mixed-form transport over a caller-provided scratch (no allocation): with
+// seg_per_iter = 0 bundles of at most kExternalBundle packets, else wavefront
+// passes over two record buffers of kExternalQueue packets each, without
+// re-sort; external_scratch_bytes() is what either needs.
+constexpr int64_t kExternalBundle = 1 << 20, kExternalKeys = 1 << 19, kExternalQueue = 1 << 16;
+constexpr int64_t external_scratch_bytes() {
+  return 2 * kExternalQueue * (32 + 8 * CRASH_MAX_BINS) > 12 * kExternalBundle + 8 * kExternalKeys + 4096
+             ? 2 * kExternalQueue * (32 + 8 * CRASH_MAX_BINS) : 12 * kExternalBundle + 8 * kExternalKeys + 4096;
+}
+int launch_trace_mixed_external(StepArgs a, const BinTables& t, const crash_run_opts& o,
+                                char* scratch, unsigned* count, int max_iter, cudaStream_t s);
 // cross sections, heating weights and heat exponent of a bin table (host)
 void cross_sections(int nb, const double* E, BinTables& t, int& heatF);
 
-// wavefront workspace (mixed form): capacity in packets, number of sort keys
-void* wavefront_create(int64_t capacity, int64_t n_keys, int n_bins, cudaError_t* err);
+// Mixed-form workspace: packets of the queue, packets of a bundle chunk, sort
+// keys of the queue's passes and direction keys of the bundles.
+struct WFSize {
+  int64_t queue = 0, bundle = 0, n_keys = 0, bundle_keys = 0;
+};
+void* wavefront_create(const WFSize& n, int n_bins, cudaError_t* err);
 void wavefront_destroy(void* w);
-int64_t wavefront_capacity(void* w);
+WFSize wavefront_size(void* w);
+// the largest number of direction keys the bundle sort scans
+constexpr int64_t kMaxBundleKeys = (int64_t)4096 * 1024;
+// threads the direct form keeps resident on the whole GPU
+int64_t resident_packets();

@@ -9,19 +9,30 @@
 // heating energy are accumulated in FP32 over the bins and rounded once per
 // cell, H I taking the remainder.
 //
-// Two launch shapes:
-//   * one thread per packet (opts.wavefront = 0): emit and trace to the end;
-//   * wavefront (default): the emission kernel writes every packet to a
+// Three forms (transport_form chooses; deposits are integer sums, so the
+// order packets are traced in never changes a result):
+//   * emission order (FORM_DIRECT): one thread per packet, emitted and traced
+//     to the end;
+//   * bundles (FORM_BUNDLE): the packets are first sorted by source and
+//     direction cell (a counting sort of packet ids), and each warp traces 32
+//     neighbouring directions of one source to the end.  The lanes of a warp
+//     stay within a few cells of one another: their gathers share sectors,
+//     their deposits in one cell are summed before they are sent, they take
+//     the same branches (thin or thick cells, which colours are left) and end
+//     together.  128^3, 1000 sources, 2e8 packets, 8 colours (1.61e10
+//     crossings): 244 ms against 383 ms for passes of the same walk;
+//   * passes (FORM_PASSES): the emission kernel writes every packet to a
 //     device queue; pass kernels (persistent, grid-stride over the live
 //     count held in device memory) advance the queue S steps at a time until
-//     it is empty.  Every
-//     R passes the queue is re-sorted by Morton order of its 8^3-cell bucket
-//     and direction octant (one-pass counting sort), so that the packets a
-//     warp holds gather neighbouring cells.  Deposits are integer sums, so
-//     the processing order never changes a result.
-// The launch sequence depends only on the grid sizes and S, never on data,
+//     it is empty.  Every R passes the queue is re-sorted by Morton order of
+//     its 8^3-cell bucket and direction (one-pass counting sort), so that the
+//     packets in flight, not only those of a warp, work on one part of a grid
+//     that does not fit L2.
+// The launch sequence depends only on sizes and options, never on data,
 // so a step is capturable in a CUDA graph.
 #include <math.h>
+
+#include <algorithm>
 
 #include "crash_internal.cuh"
 #include "k_device.cuh"
@@ -47,6 +58,8 @@ struct WF {
   uint2* items = nullptr;                // work items of a tile pass (tile, first position)
   unsigned* gsync = nullptr;             // [2] grid barrier of the persistent launch
   int64_t n_keys = 0;
+  int64_t bcap = 0;                      // packets of a bundle chunk
+  int64_t bkeys = 0;                     // direction keys of a bundle chunk
 };
 
 struct WFArgs {
@@ -76,6 +89,13 @@ __device__ __forceinline__ int64_t next_block_packets(unsigned* work) {
   if (threadIdx.x == 0) s_base = atomicAdd(work, (unsigned)blockDim.x);
   __syncthreads();
   return (int64_t)s_base;
+}
+
+// The same for a warp: the next 32 packets.
+__device__ __forceinline__ int64_t next_warp_packets(unsigned* work) {
+  unsigned base = 0;
+  if ((threadIdx.x & 31) == 0) base = atomicAdd(work, 32u);
+  return (int64_t)__shfl_sync(0xFFFFFFFFu, base, 0);
 }
 
 struct Tally {
@@ -225,14 +245,9 @@ __device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
 
 enum { ALIVE = 0, ABSORBED = 1, ESCAPED = 2 };
 
-// One bin's absorbed count once its optical depth tau and the series value
-// q = Nf (1 - e^-tau)/tau (tau < 0.5) are known: the same rounding as
-// absorb(), with the transmitted part taken for tau >= 0.5 (q replaced).
-__device__ __forceinline__ unsigned absorb_lane(unsigned m, float Nf, float tau, float& q) {
-  if (tau < 0.5f) {
-    const unsigned A = __float2uint_rn(q * tau);
-    return A > m ? m : A;
-  }
+// One bin of optical depth tau >= 0.5: the transmitted part is rounded and
+// the absorbed count is the rest, as in absorb(); q is replaced.
+__device__ __forceinline__ unsigned absorb_thick(unsigned m, float Nf, float tau, float& q) {
   const float T = Nf * expf(-tau);
   q = (Nf - T) * __fdividef(1.0f, tau);
   unsigned Np = __float2uint_rn(T);
@@ -253,11 +268,16 @@ __device__ __forceinline__ unsigned absorb_lane(unsigned m, float Nf, float tau,
 // sum_s t_s sum_j q_j (sigma w)_s,j; per bin pair that is one packed fma per
 // sum.
 //
-// THIN: every bin of the cell has tau < 0.5 (known from one bound for the
-// whole cell), so every bin takes the series and A = rint(m (1 - e^-tau))
-// needs no clamp: it is at most 0.4 m + 1/2, below m for m >= 1, so a bin
-// that held photons still holds some and the packet's liveness is unchanged
-// (left is not recomputed).
+// A bin with tau < 0.5 takes the series, and A = rint(m (1 - e^-tau)) needs
+// no clamp: it is at most 0.4 m + 1/2, below m for m >= 1, so a bin that held
+// photons still holds some.  THIN: no lane of the warp crosses a cell where
+// some bin may have tau >= 0.5 (known from one bound for the whole cell): no
+// bin is looked at on its own, and the packet's liveness is unchanged (left
+// is not recomputed).  Otherwise every bin pair is done by the series first
+// and its bins with tau >= 0.5, if any lane has some, are done again, so that
+// lanes in thin and in thick cells share one instruction stream; and a pair
+// that holds no photons in any lane (soft bins die within the first thick
+// cells) is left out: it absorbs nothing and adds nothing.
 template <int NBT, bool HE, bool HEAT, bool THIN>
 __device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 tHeI2, const f32x2 tHeII2,
                                                   Content<NBT>& c, const BinTables& t,
@@ -266,6 +286,8 @@ __device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 
   if (!THIN) left = 0;
 #pragma unroll
   for (int j = 0; j < NBT; j += 2) {
+    const unsigned m0 = c.m[j], m1 = c.m[j + 1];
+    if (!THIN && (m0 | m1) == 0u) continue;
     const f32x2 s0 = f2(t.sigma32[0][j], t.sigma32[0][j + 1]);
     f32x2 tau = f2_mul(tHI2, s0);
     f32x2 s1 = 0ull, s2 = 0ull;
@@ -274,7 +296,6 @@ __device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 
       s2 = f2(t.sigma32[2][j], t.sigma32[2][j + 1]);
       tau = f2_fma(tHeII2, s2, f2_fma(tHeI2, s1, tau));
     }
-    const unsigned m0 = c.m[j], m1 = c.m[j + 1];
     const float N0 = __uint2float_rn(m0), N1 = __uint2float_rn(m1);
     // (1 - e^-tau)/tau by the same Horner steps as absorbed_over_tau
     f32x2 p = f2(CRASH_AOT_C5, CRASH_AOT_C5);
@@ -286,24 +307,23 @@ __device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 
     f32x2 q2 = f2_mul(f2(N0, N1), p);
     // a bin with no photons or no optical depth absorbs nothing and adds
     // nothing below (q = 0 or sigma = 0), as when the scalar form skips it
-    unsigned A0, A1;
-    if (THIN) {
-      float qt0, qt1;
-      f2_split(f2_mul(q2, tau), qt0, qt1);
-      A0 = __float2uint_rn(qt0);
-      A1 = __float2uint_rn(qt1);
-    } else {
-      float tau0, tau1, q0, q1;
+    float qt0, qt1;
+    f2_split(f2_mul(q2, tau), qt0, qt1);
+    unsigned A0 = __float2uint_rn(qt0), A1 = __float2uint_rn(qt1);
+    if (!THIN) {
+      float tau0, tau1;
       f2_split(tau, tau0, tau1);
-      f2_split(q2, q0, q1);
-      A0 = absorb_lane(m0, N0, tau0, q0);
-      A1 = absorb_lane(m1, N1, tau1, q1);
-      q2 = f2(q0, q1);
+      if (fmaxf(tau0, tau1) >= 0.5f) {
+        float q0, q1;
+        f2_split(q2, q0, q1);
+        if (tau0 >= 0.5f) A0 = absorb_thick(m0, N0, tau0, q0);
+        if (tau1 >= 0.5f) A1 = absorb_thick(m1, N1, tau1, q1);
+        q2 = f2(q0, q1);
+      }
     }
     c.m[j] = m0 - A0;
     c.m[j + 1] = m1 - A1;
-    At += A0;
-    At += A1;
+    At += (unsigned long long)A0 + A1;
     if (!THIN) left |= (m0 - A0) | (m1 - A1);
     if (HE) {
       g1 = f2_fma(q2, s1, g1);
@@ -334,21 +354,20 @@ __device__ __forceinline__ void cell_shares(unsigned long long At, int e, float 
                                             float G1, float G2, float H0, float H1, float H2,
                                             long long& dHI, long long& dHeI, long long& dHeII,
                                             long long& dE) {
-  long long a1 = 0, a2 = 0, h = 0;
+  // (with At = 0 the caller sends nothing, whatever comes out here)
   const long long Au = (long long)(At << e);
-  if (At) {
-    const float unit = __uint_as_float((unsigned)(127 + e) << 23);
-    const float fHeI = HE ? tHeI * G1 : 0.f, fHeII = HE ? tHeII * G2 : 0.f;
-    const float fheat = HEAT ? (HE ? fmaf(tHeII, H2, fmaf(tHeI, H1, tHI * H0)) : tHI * H0) : 0.f;
-    round_shares(Au, fHeI * unit, fHeII * unit, fheat * unit, a1, a2, h);
-    if (!HE) a1 = a2 = 0;
-    if (!HEAT) h = 0;
-    // He shares above the cell's total only by rounding: clamp then (the
-    // clamps change nothing when the two fit)
-    if (HE && (unsigned long long)a1 + (unsigned long long)a2 > (unsigned long long)Au) {
-      a1 = a1 > Au ? Au : a1;
-      a2 = a2 > Au - a1 ? Au - a1 : a2;
-    }
+  const float unit = __uint_as_float((unsigned)(127 + e) << 23);
+  const float fHeI = HE ? tHeI * G1 : 0.f, fHeII = HE ? tHeII * G2 : 0.f;
+  const float fheat = HEAT ? (HE ? fmaf(tHeII, H2, fmaf(tHeI, H1, tHI * H0)) : tHI * H0) : 0.f;
+  long long a1, a2, h;
+  round_shares(Au, fHeI * unit, fHeII * unit, fheat * unit, a1, a2, h);
+  if (!HE) a1 = a2 = 0;
+  if (!HEAT) h = 0;
+  // He shares above the cell's total only by rounding: clamp then (the
+  // clamps change nothing when the two fit)
+  if (HE && (unsigned long long)a1 + (unsigned long long)a2 > (unsigned long long)Au) {
+    a1 = a1 > Au ? Au : a1;
+    a2 = a2 > Au - a1 ? Au - a1 : a2;
   }
   dHeI = a1;
   dHeII = a2;
@@ -373,7 +392,8 @@ __device__ __forceinline__ long long cell_attenuate_x2(float seg, float dl, floa
   // largest cross sections in the same operation order (rounding is monotone)
   const float k0max = tHI * t.sigma32_max[0];
   const float tau_max = HE ? fmaf(tHeII, t.sigma32_max[2], fmaf(tHeI, t.sigma32_max[1], k0max)) : k0max;
-  if (tau_max < 0.5f)
+  // (either form gives a lane in a thin cell the same bits: the vote only picks the instruction stream)
+  if (!__any_sync(__activemask(), !(tau_max < 0.5f)))
     attenuate_bins_x2<NBT, HE, HEAT, true>(tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
   else
     attenuate_bins_x2<NBT, HE, HEAT, false>(tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
@@ -437,19 +457,25 @@ __device__ __forceinline__ long long cell_attenuate(float seg, float dl, float4 
 //
 // The four int64 deposits of a crossing are one 32-byte record (one sector).
 // A warp sends the records of its lanes together: every lane stores its
-// record to the warp's staging area in shared memory, and the warp then walks
-// the 32 records in four steps of eight, four lanes to a record, each lane
-// adding one of its int64 values with one reduction.  The four lanes of a
-// record address one sector, so a step is one warp instruction of eight
-// sectors.  Sending a record per lane takes 32 sectors per instruction (four
-// plain reductions) or, as a 32-byte bulk reduction, one issue per lane with
-// its addresses moved to uniform registers (about 8.6 warp instructions per
-// record).  Integer sums do not depend on their order, so the deposits are
-// the same bits in every form.
+// record and its cell to the warp's staging area in shared memory, and four
+// lanes then take four neighbouring records, each lane one of the four values:
+// it adds up those of equal cells (bundles: neighbouring lanes are often in
+// one cell) and sends each sum with one reduction.  The four lanes of a record
+// address one sector, so one warp instruction sends eight records over eight
+// sectors.  Where some four records were one cell's, the sums of equal cells
+// are also merged across the warp (near a source all 32 lanes are in one
+// cell, and as many reductions of one address are serial in L2).  Sending a
+// record per lane takes 32 sectors per instruction (four plain reductions) or,
+// as a 32-byte bulk reduction, one issue per lane with its addresses moved to
+// uniform registers (about 8.6 warp instructions per record).  Passes over the
+// thin 256^3 case (3.2e7 packets): bulk reductions 123.5 ms, records sent
+// together 107.6, equal cells merged 102.7; one central source, 64^3, bundles
+// of 6.7e6 packets: 8.2 ms, merged 6.7.  Integer sums do not depend on their
+// order, so the deposits are the same bits in every form.
 constexpr int kMaxWarps = 8;             // 256 threads: the kernels' launch bound
-constexpr int kStageHalf = 576;          // second half-records: 512 bytes on, and 64 more so that the
-                                         // read below touches every bank once per half warp
-constexpr int kStageWarp = kStageHalf + 512;
+constexpr int kStageHalf = 656;          // 512 bytes of first half-records, 32 more after every 8, and 16: the
+constexpr int kStageCells = 2 * kStageHalf - 16;   // reads below then touch every bank once per half warp
+constexpr int kStageWarp = kStageCells + 128;
 
 // with a single deposited value per crossing (pure H, isothermal) the record
 // has one nonzero: each lane then sends its own
@@ -458,42 +484,75 @@ struct GlobalCells {
   static constexpr bool kWarp = true;
   const float4* abs;
   unsigned long long* dep;
-  int64_t coff;
-  int nx, ny;
+  unsigned coff, ny, nz;         // ny, nz: cells from a row, and from a plane, to the next
   unsigned char* stage;          // this warp's staging area (shared)
-  __device__ __forceinline__ int64_t index(int ix, int iy, int iz) const {
-    return coff + (ix + nx * (iy + ny * iz));
+  // cells of all boxes together are below 2^32 (their state alone is 84 bytes a cell)
+  __device__ __forceinline__ unsigned index(int ix, int iy, int iz) const {
+    return coff + (unsigned)ix + ny * (unsigned)iy + nz * (unsigned)iz;
   }
-  __device__ __forceinline__ float4 load(int64_t c) const { return __ldg(abs + c); }
+  __device__ __forceinline__ float4 load(unsigned c) const { return __ldg(abs + c); }
   // called by the whole warp; has: this lane has a record for cell c
-  __device__ __forceinline__ void add(bool has, int64_t c, long long a0, long long a1, long long a2,
+  __device__ __forceinline__ void add(bool has, unsigned c, long long a0, long long a1, long long a2,
                                       long long e) const {
     if (!HE && !HEAT) {
-      if (has) atomicAdd(dep + 4 * c, (unsigned long long)a0);
+      // neighbouring lanes in one cell (near a source) send one sum
+      unsigned cur = has ? c : 0xFFFFFFFFu;
+      unsigned long long v = (unsigned long long)a0;
+      unsigned other = __shfl_xor_sync(0xFFFFFFFFu, cur, 1);
+      if (__any_sync(0xFFFFFFFFu, has && other == cur)) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          if (o > 1) other = __shfl_xor_sync(0xFFFFFFFFu, cur, o);
+          const unsigned long long u = __shfl_xor_sync(0xFFFFFFFFu, v, o);
+          if (other == cur) {
+            if (threadIdx.x & o) cur = 0xFFFFFFFFu;
+            else v += u;
+          }
+        }
+      }
+      if (cur != 0xFFFFFFFFu) atomicAdd(dep + 4 * (size_t)cur, v);
       return;
     }
-    const unsigned mask = __ballot_sync(0xFFFFFFFFu, has);
-    if (mask == 0u) return;
+    if (!__any_sync(0xFFFFFFFFu, has)) return;
+    constexpr unsigned none = 0xFFFFFFFFu;
     const unsigned lane = threadIdx.x & 31;
-    if (has) {
-      *reinterpret_cast<ulonglong2*>(stage + 16 * lane) = make_ulonglong2((unsigned long long)a0, (unsigned long long)a1);
-      *reinterpret_cast<ulonglong2*>(stage + kStageHalf + 16 * lane) =
-          make_ulonglong2((unsigned long long)a2, (unsigned long long)e);
-    }
+    unsigned char* mine = stage + 16 * lane + 32 * (lane >> 3);
+    reinterpret_cast<unsigned*>(stage + kStageCells)[lane] = has ? c : none;
+    *reinterpret_cast<ulonglong2*>(mine) = make_ulonglong2((unsigned long long)a0, (unsigned long long)a1);
+    *reinterpret_cast<ulonglong2*>(mine + kStageHalf) = make_ulonglong2((unsigned long long)a2, (unsigned long long)e);
     __syncwarp();
-    const unsigned k = lane & 3u, r0 = lane >> 2;
-    const unsigned char* src = stage + (k >> 1) * kStageHalf + 8 * (k & 1u) + 16 * r0;
+    const unsigned k = lane & 3u, g = lane >> 2;     // value k of records 4 g .. 4 g + 3
+    const uint4 cs = *reinterpret_cast<const uint4*>(stage + kStageCells + 16 * g);
+    const unsigned char* src = stage + (k >> 1) * kStageHalf + 8 * (k & 1u) + 64 * g + 32 * (g >> 1);
+    const unsigned cq[4] = {cs.x, cs.y, cs.z, cs.w};
     unsigned long long* dk = dep + k;
-    // cells of all boxes together are below 2^32 (their state alone is 84 bytes a cell)
-    const unsigned c32 = (unsigned)c;
+    unsigned cur = cs.x;
+    unsigned long long acc = *reinterpret_cast<const unsigned long long*>(src);
+    bool whole = true;
 #pragma unroll
-    for (unsigned q = 0; q < 4; ++q) {
-      const unsigned rc = __shfl_sync(0xFFFFFFFFu, c32, 8 * q + r0);
-      if ((mask >> (8 * q + r0)) & 1u) {
-        const unsigned long long v = *reinterpret_cast<const unsigned long long*>(src + 128 * q);
-        if (v) atomicAdd(dk + 4 * (size_t)rc, v);
+    for (int q = 1; q < 4; ++q) {
+      const unsigned long long v = *reinterpret_cast<const unsigned long long*>(src + 16 * q);
+      if (cq[q] == cur) {
+        acc += v;
+      } else {
+        if (cur != none && acc) atomicAdd(dk + 4 * (size_t)cur, acc);
+        cur = cq[q];
+        acc = v;
+        whole = false;
       }
     }
+    if (__any_sync(0xFFFFFFFFu, whole)) {
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) {
+        const unsigned other = __shfl_xor_sync(0xFFFFFFFFu, cur, o);
+        const unsigned long long v = __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+        if (other == cur) {
+          if (lane & o) cur = none;
+          else acc += v;
+        }
+      }
+    }
+    if (cur != none && acc) atomicAdd(dk + 4 * (size_t)cur, acc);
     __syncwarp();                // the next crossing's records overwrite the staging area
   }
 };
@@ -505,14 +564,15 @@ struct GlobalCells {
 // over the banks), and go to the grid once per work item
 struct TileCells {
   static constexpr bool kWarp = false;
+  static constexpr unsigned ny = 16, nz = 256;
   const float4* sabs;              // shared, [16][16][16]
   unsigned long long* sdep;        // shared, [4][16][16][16]
   int x0, y0, z0;
-  __device__ __forceinline__ int64_t index(int ix, int iy, int iz) const {
-    return (ix - x0) + 16 * ((iy - y0) + 16 * (iz - z0));
+  __device__ __forceinline__ unsigned index(int ix, int iy, int iz) const {
+    return (unsigned)((ix - x0) + 16 * ((iy - y0) + 16 * (iz - z0)));
   }
-  __device__ __forceinline__ float4 load(int64_t c) const { return sabs[c]; }
-  __device__ __forceinline__ void add(bool has, int64_t c, long long a0, long long a1, long long a2,
+  __device__ __forceinline__ float4 load(unsigned c) const { return sabs[c]; }
+  __device__ __forceinline__ void add(bool has, unsigned c, long long a0, long long a1, long long a2,
                                       long long e) const {
     if (!has) return;
     if (a0) atomicAdd(sdep + c, (unsigned long long)a0);
@@ -522,119 +582,116 @@ struct TileCells {
   }
 };
 
+// The cells a walk stays in: [x0, x1) x [y0, y1) x [z0, z1).
+struct Region {
+  int x0, y0, z0, x1, y1, z1;
+};
+
 // Advance one packet by at most max_iter DDA steps.  tM* are the distances
 // (in cells, along the ray) from the current point to the next x/y/z face;
 // they are re-based at every step so that FP32 keeps their precision.  The
 // walk does not depend on the attenuation, so the next cell's absorbers are
 // requested before the current cell's bins are processed (one step of
-// software pipelining hides most of the gather latency).  With TILE the walk
-// also stops (alive) when it steps out of the box [tx0,tx0+ex) x ... .
-// With PER, a box flagged periodic wraps the walk at its faces and ends it
-// (ESCAPED) once the path trem (cells, the rest of c dt) is used up, the
-// last segment cut there (Sec. 2 periodic boxes).  The photons the walk
-// absorbed are counted once at its end, as the drop of the packet's content.
+// software pipelining hides most of the gather latency).  The walk counts the
+// cells left to the region's faces along each axis: it ends (alive, or ESCAPED
+// from the grid) when one count is used up, and the packet's cell is made from
+// the counts at the end, which takes fewer instructions per step than keeping
+// and testing the three cell indices.  With PER, a box flagged periodic wraps
+// the walk at its faces and ends it (ESCAPED) once the path trem (cells, the
+// rest of c dt) is used up, the last segment cut there (Sec. 2 periodic
+// boxes).  The photons the walk absorbed are counted once at its end, as the
+// drop of the packet's content.
 // run: the lane has a packet.  With Cells::kWarp the whole warp walks
 // together (every lane calls, and lanes whose packet is done wait for the
 // last) because the warp sends its deposits together.
-template <int NBT, bool HE, bool HEAT, bool TILE, bool PER, class Cells>
+template <int NBT, bool HE, bool HEAT, bool PER, class Cells>
 __device__ __forceinline__ int walk_steps(const bool run, int& ix, int& iy, int& iz, float& tMx, float& tMy, float& tMz,
                                     const float dx, const float dy, const float dz, Content<NBT>& N,
-                                    const BoxMeta* M, const Cells& cells, const BinTables& t,
-                                    const int nb, const int max_iter, Tally& tl, int tx0 = 0,
-                                    int ty0 = 0, int tz0 = 0, int ex = 0, int ey = 0, int ez = 0,
-                                    float* trem = nullptr) {
+                                    const BoxMeta* M, const Region& R, const Cells& cells, const BinTables& t,
+                                    const int nb, const int max_iter, Tally& tl, float* trem) {
   if (max_iter <= 0) return ALIVE;
-  const int nx = M->nx, ny = M->ny, nz = M->nz;
   const bool per = PER && M->periodic;
   const float tDx = dx != 0.f ? 1.0f / fabsf(dx) : INFINITY;
   const float tDy = dy != 0.f ? 1.0f / fabsf(dy) : INFINITY;
   const float tDz = dz != 0.f ? 1.0f / fabsf(dz) : INFINITY;
-  const int sx = dx > 0.f ? 1 : -1, sy = dy > 0.f ? 1 : -1, sz = dz > 0.f ? 1 : -1;
   const float dl = M->dlf;
   const bool heat_box = HEAT && !M->isothermal;
   unsigned left = 0;
 #pragma unroll
   for (int j = 0; j < (NBT > 0 ? NBT : CRASH_MAX_BINS); ++j)
     if (NBT > 0 || j < nb) left |= N.m[j];
-  // current segment
-  float seg = fminf(tMx, fminf(tMy, tMz));
-  int ax = (tMx <= tMy && tMx <= tMz) ? 0 : (tMy <= tMz ? 1 : 2);
-  int64_t cell = 0;
+  // steps to the region's faces, and from a cell to the next along each axis
+  int rx = dx > 0.f ? R.x1 - ix : ix - R.x0 + 1;
+  int ry = dy > 0.f ? R.y1 - iy : iy - R.y0 + 1;
+  int rz = dz > 0.f ? R.z1 - iz : iz - R.z0 + 1;
+  const unsigned stx = dx > 0.f ? 1u : ~0u, sty = dy > 0.f ? cells.ny : 0u - cells.ny,
+                 stz = dz > 0.f ? cells.nz : 0u - cells.nz;
+  unsigned next = 0;
   float4 ab = make_float4(0.f, 0.f, 0.f, 0.f);
-  bool go = run;
-  int status = ALIVE;
+  bool go = run, cut = false;
   if (go) {
-    cell = cells.index(ix, iy, iz);
-    ab = cells.load(cell);
+    next = cells.index(ix, iy, iz);
+    ab = cells.load(next);
   }
   for (int it = 1;; ++it) {
-    if (Cells::kWarp ? !__any_sync(0xFFFFFFFFu, go) : !go) return status;
-    const int64_t at = cell;
+    if (Cells::kWarp ? !__any_sync(0xFFFFFFFFu, go) : !go) break;
+    const unsigned cell = next;
     bool has = false;
     long long dHI = 0, dHeI = 0, dHeII = 0, dE = 0;
     if (go) {
-      // step the walk into the next cell and request its absorbers
-      const bool bx = ax == 0, by = ax == 1, bz = ax == 2;
+      // step the walk into the next cell (ties x before y before z) and
+      // request its absorbers
+      float seg = fminf(tMx, fminf(tMy, tMz));
+      const bool bx = tMx == seg, by = !bx && tMy == seg, bz = !bx && !by;
       tMx = bx ? tDx : tMx - seg;
       tMy = by ? tDy : tMy - seg;
       tMz = bz ? tDz : tMz - seg;
-      ix += bx ? sx : 0;
-      iy += by ? sy : 0;
-      iz += bz ? sz : 0;
-      if (PER && per) {
-        ix = ix < 0 ? nx - 1 : (ix >= nx ? 0 : ix);
-        iy = iy < 0 ? ny - 1 : (iy >= ny ? 0 : iy);
-        iz = iz < 0 ? nz - 1 : (iz >= nz ? 0 : iz);
+      rx -= bx ? 1 : 0;
+      ry -= by ? 1 : 0;
+      rz -= bz ? 1 : 0;
+      next += bx ? stx : (by ? sty : stz);
+      bool leave = min(rx, min(ry, rz)) == 0;
+      if (PER && per && leave) {
+        // back in through the opposite face
+        if (rx == 0) { rx = R.x1 - R.x0; next -= stx * (unsigned)rx; }
+        if (ry == 0) { ry = R.y1 - R.y0; next -= sty * (unsigned)ry; }
+        if (rz == 0) { rz = R.z1 - R.z0; next -= stz * (unsigned)rz; }
+        leave = false;
       }
-      const bool out = ((unsigned)ix >= (unsigned)nx) | ((unsigned)iy >= (unsigned)ny) |
-                       ((unsigned)iz >= (unsigned)nz);
-      const bool leave = TILE ? (((unsigned)(ix - tx0) >= (unsigned)ex) | ((unsigned)(iy - ty0) >= (unsigned)ey) |
-                                 ((unsigned)(iz - tz0) >= (unsigned)ez))
-                              : out;
-      float seg_n = 0.f;
-      int ax_n = 0;
-      float4 ab_n = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (!leave) {
-        seg_n = fminf(tMx, fminf(tMy, tMz));
-        ax_n = (tMx <= tMy && tMx <= tMz) ? 0 : (tMy <= tMz ? 1 : 2);
-        cell = cells.index(ix, iy, iz);
-        ab_n = cells.load(cell);
-      }
+      const float4 here = ab;
+      if (!leave) ab = cells.load(next);
       // periodic: the path left to the light-travel distance cuts the segment
-      bool stop = false;
       if (PER && per) {
-        stop = seg >= *trem;
-        if (stop) seg = *trem;
+        cut = seg >= *trem;
+        if (cut) seg = *trem;
         *trem -= seg;
       }
-      if (PER && stop) { go = false; status = ESCAPED; }
-      else if (out) { go = false; status = ESCAPED; }
-      else if ((TILE && leave) || it >= max_iter) go = false;
-      // attenuate and deposit in the current cell
-      if (seg > 0.f) {
-        has = cell_attenuate<NBT, HE, HEAT>(seg, dl, ab, N, nb, t, dHI, dHeI, dHeII, dE, left) != 0;
-        tl.crossings += 1;
-        if (left == 0) { go = false; status = ABSORBED; }
-        if (!heat_box) dE = 0;
-      }
-      seg = seg_n;
-      ax = ax_n;
-      ab = ab_n;
+      go = !(leave || it >= max_iter || (PER && cut));
+      // attenuate and deposit in the current cell (a segment of no length
+      // absorbs nothing and is no crossing)
+      has = cell_attenuate<NBT, HE, HEAT>(seg, dl, here, N, nb, t, dHI, dHeI, dHeII, dE, left) != 0;
+      tl.crossings += seg > 0.f ? 1u : 0u;
+      if (left == 0 && seg > 0.f) go = false;
+      if (!heat_box) dE = 0;
     }
-    cells.add(has, at, dHI, dHeI, dHeII, dE);
+    cells.add(has, cell, dHI, dHeI, dHeII, dE);
   }
+  ix = dx > 0.f ? R.x1 - rx : R.x0 + rx - 1;
+  iy = dy > 0.f ? R.y1 - ry : R.y0 + ry - 1;
+  iz = dz > 0.f ? R.z1 - rz : R.z0 + rz - 1;
+  if (left == 0) return ABSORBED;
+  const bool out = ((unsigned)ix >= (unsigned)M->nx) | ((unsigned)iy >= (unsigned)M->ny) | ((unsigned)iz >= (unsigned)M->nz);
+  return out || (PER && cut) ? ESCAPED : ALIVE;
 }
 
-template <int NBT, bool HE, bool HEAT, bool TILE, bool PER, class Cells>
+template <int NBT, bool HE, bool HEAT, bool PER, class Cells>
 __device__ __forceinline__ int walk(const bool run, int& ix, int& iy, int& iz, float& tMx, float& tMy, float& tMz,
                                     const float dx, const float dy, const float dz, Content<NBT>& N,
-                                    const BoxMeta* M, const Cells& cells, const BinTables& t,
-                                    const int nb, const int max_iter, Tally& tl, int tx0 = 0,
-                                    int ty0 = 0, int tz0 = 0, int ex = 0, int ey = 0, int ez = 0,
-                                    float* trem = nullptr) {
+                                    const BoxMeta* M, const Region& R, const Cells& cells, const BinTables& t,
+                                    const int nb, const int max_iter, Tally& tl, float* trem = nullptr) {
   if (run) tl.absorbed += N.total(nb);
-  const int r = walk_steps<NBT, HE, HEAT, TILE, PER>(run, ix, iy, iz, tMx, tMy, tMz, dx, dy, dz, N, M, cells, t,
-                                                     nb, max_iter, tl, tx0, ty0, tz0, ex, ey, ez, trem);
+  const int r = walk_steps<NBT, HE, HEAT, PER>(run, ix, iy, iz, tMx, tMy, tMz, dx, dy, dz, N, M, R, cells, t,
+                                               nb, max_iter, tl, trem);
   if (run) tl.absorbed -= N.total(nb);
   return r;
 }
@@ -648,10 +705,11 @@ __device__ __forceinline__ int trace_mixed(const bool run, int& ix, int& iy, int
                                            const StepArgs& a, const BinTables& t, const int nb,
                                            const int max_iter, Tally& tl, float* trem = nullptr) {
   __shared__ __align__(16) unsigned char stage[(HE || HEAT) ? kMaxWarps * kStageWarp : 16];
-  const GlobalCells<HE, HEAT> cells{reinterpret_cast<const float4*>(a.abs32), a.dep, M->cell_off, M->nx, M->ny,
+  const GlobalCells<HE, HEAT> cells{reinterpret_cast<const float4*>(a.abs32), a.dep, (unsigned)M->cell_off,
+                                    (unsigned)M->nx, (unsigned)M->nx * (unsigned)M->ny,
                                     stage + ((HE || HEAT) ? (threadIdx.x >> 5) * kStageWarp : 0)};
-  return walk<NBT, HE, HEAT, false, PER>(run, ix, iy, iz, tMx, tMy, tMz, dx, dy, dz, N, M, cells, t,
-                                         nb, max_iter, tl, 0, 0, 0, 0, 0, 0, trem);
+  const Region R{0, 0, 0, M->nx, M->ny, M->nz};
+  return walk<NBT, HE, HEAT, PER>(run, ix, iy, iz, tMx, tMy, tMz, dx, dy, dz, N, M, R, cells, t, nb, max_iter, tl, trem);
 }
 
 // warp-aggregated append of surviving packets to the output queue
@@ -668,15 +726,46 @@ __device__ __forceinline__ long long append_slot(bool alive, unsigned* count_out
   return (long long)base + __popc(m & ((1u << lane) - 1u));
 }
 
-// sort key: the packet's 8^3-cell bucket (16^3-cell tile for tile passes)
-// along the Morton or Hilbert curve, then its direction octant
+__device__ __forceinline__ unsigned spread_bits2(unsigned v) {   // 16 bits -> every second bit
+  v = (v | (v << 8)) & 0x00FF00FFu;
+  v = (v | (v << 4)) & 0x0F0F0F0Fu;
+  v = (v | (v << 2)) & 0x33333333u;
+  v = (v | (v << 1)) & 0x55555555u;
+  return v;
+}
+
+// position of a direction on a Morton curve over the octahedral map of the
+// sphere (the octahedron |x| + |y| + |z| = 1 with its lower half folded out),
+// 2^bits cells on each of the square's two axes
+__device__ __forceinline__ unsigned direction_cell(float dx, float dy, float dz, int bits) {
+  const float s = 1.0f / (fabsf(dx) + fabsf(dy) + fabsf(dz));
+  float u = dx * s, v = dy * s;
+  if (dz < 0.f) {
+    const float fu = copysignf(1.0f - fabsf(v), u), fv = copysignf(1.0f - fabsf(u), v);
+    u = fu;
+    v = fv;
+  }
+  const int m = 1 << bits;
+  const int iu = min(max((int)((u * 0.5f + 0.5f) * (float)m), 0), m - 1);
+  const int iv = min(max((int)((v * 0.5f + 0.5f) * (float)m), 0), m - 1);
+  return spread_bits2((unsigned)iu) | (spread_bits2((unsigned)iv) << 1);
+}
+
+// sort key: the packet's 8^3-cell bucket along the Morton or Hilbert curve,
+// then its direction cell (16^3-cell tile, then octant, for tile passes).
+// Finer directions than octants keep the packets of a warp together over a
+// whole pass: their gathers then share sectors, and passes may be longer
+// (256^3 thin, 6e7 packets: octants 139.6 / 137.3 / 138.5 ms with passes of
+// 32 / 48 / 64 cells, 64 direction cells 135.0 / 131.5 / 131.3 ms).
 __device__ __forceinline__ unsigned sort_key(const BoxMeta* boxes, int box, int ix, int iy, int iz,
                                              float dx, float dy, float dz, int tile, int curve) {
-  const unsigned oct = (dx < 0.f ? 1u : 0u) | (dy < 0.f ? 2u : 0u) | (dz < 0.f ? 4u : 0u);
   const int sh = tile ? 4 : 3;
   const BoxMeta& M = boxes[box];
   const unsigned pos = curve_key3((unsigned)ix >> sh, (unsigned)iy >> sh, (unsigned)iz >> sh,
                                   tile ? M.tile_bits : M.bucket_bits, curve != 0);
+  if (!tile && M.dir_bits > 1)
+    return (unsigned)M.bucket_off + ((pos << (2 * M.dir_bits)) | direction_cell(dx, dy, dz, M.dir_bits));
+  const unsigned oct = (dx < 0.f ? 1u : 0u) | (dy < 0.f ? 2u : 0u) | (dz < 0.f ? 4u : 0u);
   const unsigned base = tile ? (unsigned)M.tile_off : (unsigned)M.bucket_off;
   return base + ((pos << 3) | oct);
 }
@@ -775,20 +864,27 @@ __device__ __forceinline__ void write_survivor(const StepArgs& a, const WFArgs& 
 }
 
 // ------------------------------------------------------------------ emission
+// source of the local-th packet of a box, W packets to a source
+__device__ __forceinline__ int source_in_box(int64_t local, uint32_t W) {
+  return (uint64_t)local >> 32 ? (int)(local / W) : (int)((uint32_t)local / W);
+}
+
 // MINB = 3 keeps three 256-thread blocks resident per SM (at most 85
 // registers); MINB = 4 caps the kernels at 64 registers for four.
 // Emission of the packets [g0, g0 + n) of the launch, grid-stride over the
 // calling grid: each is traced S steps (0: emission only) and, when the launch
 // keeps a queue (S < max_steps_all), written to it with its sort key.
-template <int NBT, bool HE, bool HEAT, bool PER>
+template <int NBT, bool HE, bool HEAT, bool PER, bool ORDER = false>
 __device__ __forceinline__ void emit_range(const StepArgs& a, const BinTables& t, const WFArgs& w, int64_t g0,
                                            int64_t n, int S, int max_steps_all) {
   const int nb = NBT > 0 ? NBT : t.n_bins;
   const uint32_t step = (uint32_t)*a.step_dev;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   Tally tl{0, 0, 0, 0u, 0u};
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += stride) {
-    const int64_t i = base + threadIdx.x;
+  for (int64_t base = ORDER ? next_warp_packets(w.work) : (int64_t)blockIdx.x * blockDim.x; base < n;
+       base = ORDER ? next_warp_packets(w.work) : base + stride) {
+    const int64_t j = base + (ORDER ? threadIdx.x & 31 : threadIdx.x);
+    const int64_t i = ORDER && j < n ? (int64_t)__ldg(w.perm + j) : j;
     int b = -1;
     bool alive = false;
     int ix = 0, iy = 0, iz = 0;
@@ -803,7 +899,7 @@ __device__ __forceinline__ void emit_range(const StepArgs& a, const BinTables& t
       M = a.boxes + b;
       const int64_t local = gid - M->pkt_off;
       const uint32_t W = M->win_hi - M->win_lo;
-      const int s_local = (int)(local / W);
+      const int s_local = source_in_box(local, W);
       const uint32_t p = M->win_lo + (uint32_t)(local - (int64_t)s_local * W);
       const int s = M->src_off + s_local;
       if (!iso_direction_f32(M->seed, step, (uint32_t)s_local, p, fx, fy, fz)) {
@@ -853,6 +949,103 @@ template <int NBT, bool HE, bool HEAT, int MINB, bool PER = false>
 __global__ void __launch_bounds__(256, MINB) k_emit_mixed(StepArgs a, BinTables t, WFArgs w, int64_t g0,
                                                    int64_t n, int S, int max_steps_all) {
   emit_range<NBT, HE, HEAT, PER>(a, t, w, g0, n, S, max_steps_all);
+}
+
+// exclusive prefix sum over the block's threads
+__device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned* sh, unsigned* total) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) sh[wid] = x;
+  __syncthreads();
+  if (wid == 0) {
+    unsigned s = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned y = __shfl_up_sync(0xFFFFFFFFu, s, o);
+      if (lane >= o) s += y;
+    }
+    sh[lane] = s;
+  }
+  __syncthreads();
+  const unsigned warp_base = wid > 0 ? sh[wid - 1] : 0u;
+  *total = sh[(blockDim.x >> 5) - 1];
+  __syncthreads();
+  return warp_base + x - v;
+}
+
+// ------------------------------------------------------------------ bundles
+// key of every packet of the chunk: its source within the chunk and its
+// direction cell; the packet's rank among equal keys
+__global__ void __launch_bounds__(256) k_bundle_count(StepArgs a, unsigned* key, unsigned* rank, unsigned* bcount,
+                                                      int64_t g0, int64_t n, int s0, int bits) {
+  const uint32_t step = (uint32_t)*a.step_dev;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t gid = g0 + i;
+    const int b = box_of_packet(a.boxes, a.n_boxes, gid);
+    const BoxMeta* M = a.boxes + b;
+    const int64_t local = gid - M->pkt_off;
+    const uint32_t W = M->win_hi - M->win_lo;
+    const int s_local = source_in_box(local, W);
+    const uint32_t p = M->win_lo + (uint32_t)(local - (int64_t)s_local * W);
+    float fx = 0.f, fy = 0.f, fz = 1.f;       // (a failed draw is reported when the packet is traced)
+    iso_direction_f32(M->seed, step, (uint32_t)s_local, p, fx, fy, fz);
+    const unsigned k = ((unsigned)(M->src_off + s_local - s0) << (2 * bits)) + direction_cell(fx, fy, fz, bits);
+    key[i] = k;
+    rank[i] = atomicAdd(bcount + k, 1u);
+  }
+}
+
+// exclusive scan of the key counts, 4096 keys per block; the last block to
+// finish scans the block sums, so that the sorted position of a packet is
+// boff[key] + bsum[key / 4096] + rank
+__global__ void __launch_bounds__(1024) k_bundle_scan(const unsigned* bcount, unsigned* boff, unsigned* bsum,
+                                                      unsigned* done, int64_t n) {
+  __shared__ unsigned sh[32];
+  __shared__ bool last;
+  const int64_t base = (int64_t)blockIdx.x * 4096 + threadIdx.x * 4;
+  unsigned v[4], s = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = (base + k < n) ? bcount[base + k] : 0u;
+    s += v[k];
+  }
+  unsigned tot;
+  unsigned ex = block_excl_scan(s, sh, &tot);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (base + k < n) boff[base + k] = ex;
+    ex += v[k];
+  }
+  if (threadIdx.x == 0) {
+    bsum[blockIdx.x] = tot;
+    __threadfence();
+    last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last) return;
+  const unsigned mine = threadIdx.x < gridDim.x ? __ldcg(bsum + threadIdx.x) : 0u;
+  ex = block_excl_scan(mine, sh, &tot);
+  if (threadIdx.x < gridDim.x) bsum[threadIdx.x] = ex;
+}
+
+__global__ void __launch_bounds__(256) k_bundle_place(const unsigned* key, const unsigned* rank, const unsigned* boff,
+                                                      const unsigned* bsum, unsigned* order, int64_t n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned k = key[i];
+    order[boff[k] + bsum[k >> 12] + rank[i]] = (unsigned)i;
+  }
+}
+
+template <int NBT, bool HE, bool HEAT, bool PER>
+__global__ void __launch_bounds__(256, 4) k_trace_bundle(StepArgs a, BinTables t, WFArgs w, int64_t g0,
+                                                         int64_t n, int max_iter) {
+  emit_range<NBT, HE, HEAT, PER, true>(a, t, w, g0, n, max_iter, max_iter);
 }
 
 // One re-emission packet per entry of this step's list (diffuse
@@ -1005,32 +1198,6 @@ __device__ __forceinline__ void pass_range_q(const StepArgs& a, const BinTables&
 
 // ------------------------------------------------------------------ re-sort
 // exclusive scan of bcount into boff: 4096 keys per block, block sums, add
-__device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned* sh, unsigned* total) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  unsigned x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) sh[wid] = x;
-  __syncthreads();
-  if (wid == 0) {
-    unsigned s = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0u;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned y = __shfl_up_sync(0xFFFFFFFFu, s, o);
-      if (lane >= o) s += y;
-    }
-    sh[lane] = s;
-  }
-  __syncthreads();
-  const unsigned warp_base = wid > 0 ? sh[wid - 1] : 0u;
-  *total = sh[(blockDim.x >> 5) - 1];
-  __syncthreads();
-  return warp_base + x - v;
-}
-
 __global__ void __launch_bounds__(1024) k_scan_blocks(const unsigned* in, unsigned* out,
                                                       unsigned* bsum, int64_t n) {
   __shared__ unsigned sh[32];
@@ -1189,8 +1356,9 @@ __global__ void __launch_bounds__(kTileBlock, 1) k_tile_pass(StepArgs a, BinTabl
       if (j < hi) {
         load_record<NBT>(w.rec_in, w.rs, (long long)w.perm[j], ix, iy, iz, pb, tMx, tMy, tMz, fx, fy, fz,
                          N, nb);
-        const int r = walk<NBT, HE, HEAT, true, false>(true, ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, cells,
-                                                       t, nb, 64, tl, x0, y0, z0, ex, ey, ez);
+        const Region R{x0, y0, z0, x0 + ex, y0 + ey, z0 + ez};
+        const int r = walk<NBT, HE, HEAT, false>(true, ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, R, cells, t, nb, 64,
+                                                 tl);
         if (r == ESCAPED) tl.escaped += N.total(nb);
         alive = (r == ALIVE);
       }
@@ -1416,6 +1584,13 @@ int num_sms() {
   return g_num_sms;
 }
 
+// source (over all boxes) of a packet of the launch
+int source_of_packet(const StepArgs& a, int64_t gid) {
+  const BoxMeta* M = a.boxes_host + a.n_boxes - 1;
+  while (M->pkt_off > gid || M->pkt_count == 0) --M;
+  return M->src_off + (int)((gid - M->pkt_off) / (M->win_hi - M->win_lo));
+}
+
 template <int NBT, bool HE, bool HEAT>
 int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF* wf, int max_iter,
               cudaStream_t s, EventPairs* ev, int* ev_used) {
@@ -1438,24 +1613,16 @@ int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF
     (*ev_used)++;
   };
   if (a.total_packets <= 0) return 0;
-  if (a.any_periodic) {
-    // periodic boxes: one thread per packet, traced to the end of its c dt
-    int64_t blocks = (a.total_packets + block - 1) / block;
-    if (blocks > (int64_t)1 << 30) blocks = (int64_t)1 << 30;
-    WFArgs w = wf_args(wf, 0, false, false);
-    tic();
-    k_emit_mixed<NBT, HE, HEAT, 3, true><<<(unsigned)blocks, block, 0, s>>>(a, t, w, 0, a.total_packets,
-                                                                         max_iter, max_iter);
-    toc();
-    return 1;
-  }
-  if (!o.wavefront || wf->cap == 0) {
+  if (a.form == FORM_DIRECT) {
     // one thread per packet, traced to the end
     WFArgs w = wf_args(wf, 0, false, false);
     int64_t blocks = (a.total_packets + block - 1) / block;
     if (blocks > (int64_t)1 << 30) blocks = (int64_t)1 << 30;
     tic();
-    if (o.reg_cap)
+    if (a.any_periodic)
+      k_emit_mixed<NBT, HE, HEAT, 3, true><<<(unsigned)blocks, block, 0, s>>>(a, t, w, 0, a.total_packets,
+                                                                           max_iter, max_iter);
+    else if (o.reg_cap)
       k_emit_mixed<NBT, HE, HEAT, 4><<<(unsigned)blocks, block, 0, s>>>(a, t, w, 0, a.total_packets,
                                                                        max_iter, max_iter);
     else
@@ -1463,6 +1630,33 @@ int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF
                                                                        max_iter, max_iter);
     toc();
     return 1;
+  }
+  if (a.form == FORM_BUNDLE) {
+    for (int64_t g0 = 0; g0 < a.total_packets; g0 += wf->bcap) {
+      const int64_t n = std::min<int64_t>(wf->bcap, a.total_packets - g0);
+      // the chunk's sources, each with 4^bits direction cells: about two
+      // packets to a cell, so that the 32 packets of a warp are neighbours
+      const int s0 = source_of_packet(a, g0);
+      const int64_t ns = source_of_packet(a, g0 + n - 1) - s0 + 1;
+      int bits = 0;
+      while (bits < 11 && (ns << (2 * bits + 2)) <= std::min<int64_t>(wf->bkeys, n / 2)) ++bits;
+      const int64_t nk = ns << (2 * bits);
+      WFArgs w = wf_args(wf, 0, true, false);
+      w.work = wf->count + 2;
+      cudaMemsetAsync(wf->count, 0, 4 * sizeof(unsigned), s);
+      cudaMemsetAsync(wf->bcount, 0, sizeof(unsigned) * nk, s);
+      const unsigned nsort = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 16);
+      k_bundle_count<<<nsort, 256, 0, s>>>(a, wf->key, wf->rank, wf->bcount, g0, n, s0, bits);
+      k_bundle_scan<<<(unsigned)((nk + 4095) / 4096), 1024, 0, s>>>(wf->bcount, wf->boff, wf->bsum, wf->count + 3, nk);
+      k_bundle_place<<<nsort, 256, 0, s>>>(wf->key, wf->rank, wf->boff, wf->bsum, wf->perm, n);
+      const unsigned ntrace = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 4);
+      tic();
+      if (a.any_periodic) k_trace_bundle<NBT, HE, HEAT, true><<<ntrace, 256, 0, s>>>(a, t, w, g0, n, max_iter);
+      else k_trace_bundle<NBT, HE, HEAT, false><<<ntrace, 256, 0, s>>>(a, t, w, g0, n, max_iter);
+      toc();
+      launches += 4;
+    }
+    return launches;
   }
   if (o.tile && wf->items) {
     // emission only (no walk), then tile passes until every packet is done
@@ -1513,13 +1707,13 @@ int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF
     }
     return launches;
   }
-  const int S = o.seg_per_iter > 0 ? o.seg_per_iter : 32;
+  const int S = o.seg_per_iter > 0 ? o.seg_per_iter : 64;
   const int R = o.resort_interval == 0 ? 1 : o.resort_interval;
   // emission only writes the packets (no walk): every crossing is made by the
   // passes, which read the queue in sorted order
   int passes = (max_iter + S - 1) / S + 1;
   if (o.pass_limit > 0 && o.pass_limit < passes) passes = o.pass_limit;
-  if (o.persistent && wf->gsync) {
+  if (o.persistent && wf->gsync && !a.launch_per_pass) {
     // one cooperative launch for the whole step (all blocks resident)
     static int per_sm[2] = {0, 0};
     const int ci = o.reg_cap ? 1 : 0;
@@ -1544,6 +1738,7 @@ int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF
     return e == cudaSuccess ? 1 : -1;
   }
   const int nscan = (int)((wf->n_keys + 4095) / 4096);
+  const bool cap64 = o.reg_cap || a.launch_per_pass;
   // the pass p (p >= 1) reads in sorted order when R > 0 and p % R == 0
   auto sorted_pass = [&](int p) { return p >= 1 && p < passes && R > 0 && (p % R) == 0; };
   for (int64_t g0 = 0; g0 < a.total_packets; g0 += wf->cap) {
@@ -1563,12 +1758,12 @@ int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF
       if (p == 0) {
         int64_t blocks = (n + block - 1) / block;
         if (blocks > persistent * 4) blocks = persistent * 4;
-        if (o.reg_cap)
+        if (cap64)
           k_emit_mixed<NBT, HE, HEAT, 4><<<(unsigned)blocks, block, 0, s>>>(a, t, w, g0, n, 0, max_iter);
         else
           k_emit_mixed<NBT, HE, HEAT, 3><<<(unsigned)blocks, block, 0, s>>>(a, t, w, g0, n, 0, max_iter);
       } else {
-        if (o.reg_cap) k_pass_mixed<NBT, HE, HEAT, 4><<<persistent, block, 0, s>>>(a, t, w, S);
+        if (cap64) k_pass_mixed<NBT, HE, HEAT, 4><<<persistent, block, 0, s>>>(a, t, w, S);
         else k_pass_mixed<NBT, HE, HEAT, 3><<<persistent, block, 0, s>>>(a, t, w, S);
       }
       toc();
@@ -1615,40 +1810,61 @@ int launch_trace_mixed(const StepArgs& a, const BinTables& t, const crash_run_op
   return r;
 }
 
-int launch_trace_mixed_external(const StepArgs& a, const BinTables& t, const crash_run_opts& o,
-                                char* rec0, char* rec1, unsigned* count, int64_t cap, int max_iter,
-                                cudaStream_t s) {
+int64_t resident_packets() { return (int64_t)num_sms() * 3 * 256; }
+
+int launch_trace_mixed_external(StepArgs a, const BinTables& t, const crash_run_opts& o, char* scratch,
+                                unsigned* count, int max_iter, cudaStream_t s) {
   WF wf;                       // views the caller's buffers; owns nothing
-  wf.cap = cap;
   wf.nb = t.n_bins;
   wf.rs = ((32 + 4 * t.n_bins) + 15) / 16 * 16;
-  wf.rec[0] = rec0;
-  wf.rec[1] = rec1;
   wf.count = count;
   crash_run_opts oo = o;
   oo.wavefront = 1;
-  oo.resort_interval = -1;     // no sort keys without their workspace
   oo.tile = 0;
-  oo.persistent = 0;           // no grid barrier word either
+  if (o.seg_per_iter > 0) {
+    wf.cap = kExternalQueue;
+    wf.rec[0] = scratch;
+    wf.rec[1] = scratch + kExternalQueue * (32 + 8 * CRASH_MAX_BINS);
+    oo.resort_interval = -1;   // no sort keys without their workspace
+    oo.persistent = 0;         // no grid barrier word either
+    a.form = FORM_PASSES;
+  } else {
+    wf.bcap = kExternalBundle;
+    wf.bkeys = kExternalKeys;
+    unsigned* u = reinterpret_cast<unsigned*>(scratch);
+    wf.key = u;
+    wf.rank = u + kExternalBundle;
+    wf.perm = u + 2 * kExternalBundle;
+    wf.bcount = u + 3 * kExternalBundle;
+    wf.boff = wf.bcount + kExternalKeys;
+    wf.bsum = wf.boff + kExternalKeys;
+    a.form = a.total_packets <= resident_packets() ? FORM_DIRECT : FORM_BUNDLE;
+  }
   return launch_trace_mixed(a, t, oo, &wf, max_iter, s, nullptr, nullptr);
 }
 
-void* wavefront_create(int64_t cap, int64_t n_keys, int nb, cudaError_t* err) {
+void* wavefront_create(const WFSize& n, int nb, cudaError_t* err) {
   WF* w = new WF();
-  w->cap = cap;
+  w->cap = n.queue;
+  w->bcap = n.bundle;
+  w->bkeys = n.bundle_keys;
+  w->n_keys = n.n_keys;
   w->nb = nb;
   w->rs = ((32 + 4 * nb) + 15) / 16 * 16;
-  w->n_keys = n_keys;
+  const int64_t most = std::max(n.queue, n.bundle);
+  const int64_t keys = std::max(n.queue > 0 ? n.n_keys : (int64_t)0, n.bundle > 0 ? n.bundle_keys : (int64_t)0);
   cudaError_t e = cudaMalloc(&w->count, 4 * sizeof(unsigned));
-  if (e == cudaSuccess && cap > 0) {
-    for (int b = 0; b < 2 && e == cudaSuccess; ++b) e = cudaMalloc(&w->rec[b], (size_t)w->rs * cap);
-    if (e == cudaSuccess) e = cudaMalloc(&w->key, sizeof(unsigned) * cap);
-    if (e == cudaSuccess) e = cudaMalloc(&w->rank, sizeof(unsigned) * cap);
-    if (e == cudaSuccess) e = cudaMalloc(&w->perm, sizeof(unsigned) * cap);
-    if (e == cudaSuccess) e = cudaMalloc(&w->bcount, sizeof(unsigned) * n_keys);
-    if (e == cudaSuccess) e = cudaMalloc(&w->boff, sizeof(unsigned) * n_keys);
+  if (most > 0) {
+    if (e == cudaSuccess) e = cudaMalloc(&w->key, sizeof(unsigned) * most);
+    if (e == cudaSuccess) e = cudaMalloc(&w->rank, sizeof(unsigned) * most);
+    if (e == cudaSuccess) e = cudaMalloc(&w->perm, sizeof(unsigned) * most);
+    if (e == cudaSuccess) e = cudaMalloc(&w->bcount, sizeof(unsigned) * keys);
+    if (e == cudaSuccess) e = cudaMalloc(&w->boff, sizeof(unsigned) * keys);
     if (e == cudaSuccess) e = cudaMalloc(&w->bsum, sizeof(unsigned) * 1024);
-    if (e == cudaSuccess) e = cudaMalloc(&w->items, sizeof(uint2) * (n_keys / 8 + cap / 2048 + 2));
+  }
+  if (n.queue > 0) {
+    for (int b = 0; b < 2 && e == cudaSuccess; ++b) e = cudaMalloc(&w->rec[b], (size_t)w->rs * n.queue);
+    if (e == cudaSuccess) e = cudaMalloc(&w->items, sizeof(uint2) * (n.n_keys / 8 + n.queue / 2048 + 2));
     if (e == cudaSuccess) e = cudaMalloc(&w->gsync, 2 * sizeof(unsigned));
   }
   if (err) *err = e;
@@ -1669,7 +1885,14 @@ void wavefront_destroy(void* p) {
   delete w;
 }
 
-int64_t wavefront_capacity(void* p) { return p ? ((WF*)p)->cap : 0; }
+WFSize wavefront_size(void* p) {
+  WFSize n;
+  if (p) {
+    const WF* w = (const WF*)p;
+    n = {w->cap, w->bcap, w->n_keys, w->bkeys};
+  }
+  return n;
+}
 
 int launch_rec_mixed(const StepArgs& a, const BinTables& t, cudaStream_t s) {
   const bool he = a.any_he != 0, heat = a.any_heat != 0;

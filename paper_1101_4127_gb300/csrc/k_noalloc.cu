@@ -3,8 +3,8 @@
 // inside another framework's memory pool or under a strict memory budget,
 // plug-ins that may only use buffers handed to them, processes that must not
 // grow their footprint after start-up).  The caller passes the absorbers and
-// the deposit buffer; every scratch buffer of the step (the wavefront packet
-// queue, the per-source budget tables, the counters) lives in the file-scope
+// the deposit buffer; every scratch buffer of the step (the packet queue
+// or the sort buffers, the per-source budget tables, the counters) lives in the file-scope
 // array below, which every GPU that loads the library holds until the
 // process exits.
 #include <cuda_runtime.h>
@@ -20,14 +20,11 @@
 namespace {
 
 // capacity of the static scratch
-constexpr int64_t kQueuePackets = 1 << 16;         // packets held by each queue buffer
 constexpr int kMaxSources = CRASH_NOALLOC_MAX_SOURCES;
-constexpr int64_t kRecordBytes = 32 + 8 * CRASH_MAX_BINS;   // largest record (16 bins)
 
 constexpr int64_t align256(int64_t x) { return (x + 255) / 256 * 256; }
-constexpr int64_t kOffRec0 = 0;
-constexpr int64_t kOffRec1 = kOffRec0 + align256(kQueuePackets * kRecordBytes);
-constexpr int64_t kOffCount = kOffRec1 + align256(kQueuePackets * kRecordBytes);
+constexpr int64_t kOffWork = 0;                    // the transport's packet queue or sort buffers
+constexpr int64_t kOffCount = kOffWork + align256(external_scratch_bytes());
 constexpr int64_t kOffErr = kOffCount + 256;
 constexpr int64_t kOffStep = kOffErr + 256;
 constexpr int64_t kOffMeta = kOffStep + 256;
@@ -178,7 +175,7 @@ extern "C" crash_status crash_transport_noalloc(const crash_grid_desc* grid, int
     if (e != cudaSuccess) return fail(CRASH_ERR_CUDA, std::string("copy into scratch: ") + cudaGetErrorString(e));
   }
   // the budget of this call starts at zero; the queue counters are cleared
-  // by the wavefront launcher for every chunk
+  // by the launcher for every chunk
   {
     const cudaError_t e = cudaMemsetAsync(base + kOffBudget, 0, 64, s);
     if (e != cudaSuccess) return fail(CRASH_ERR_CUDA, std::string("clearing the budget: ") + cudaGetErrorString(e));
@@ -187,6 +184,7 @@ extern "C" crash_status crash_transport_noalloc(const crash_grid_desc* grid, int
   StepArgs a;
   memset(&a, 0, sizeof a);
   a.boxes = (const BoxMeta*)(base + kOffMeta);
+  a.boxes_host = &m;
   a.n_boxes = 1;
   a.step_dev = (unsigned long long*)(base + kOffStep);
   a.dt = dt_s;
@@ -213,8 +211,8 @@ extern "C" crash_status crash_transport_noalloc(const crash_grid_desc* grid, int
   o.chemistry = 0;
 
   launch_budget(a, t, s);
-  const int nk = launch_trace_mixed_external(a, t, o, (char*)(base + kOffRec0), (char*)(base + kOffRec1),
-                                             (unsigned*)(base + kOffCount), kQueuePackets, m.max_iter, s);
+  const int nk = launch_trace_mixed_external(a, t, o, (char*)(base + kOffWork), (unsigned*)(base + kOffCount),
+                                             m.max_iter, s);
   if (nk < 0) return fail(CRASH_ERR_CUDA, "transport launch failed");
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(CRASH_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
