@@ -708,7 +708,7 @@ static crash_status enqueue_step(crash_ctx* c, const StepArgs& a, bool timing, i
         }
         CK(cudaEventRecord(c->events[c->ev_used].first, c->stream));
       }
-      launch_trace_fp64(a, c->tables, c->opts.block_size, c->stream);
+      *nk += launch_trace_fp64(a, c->tables, c->opts.block_size, c->wf, c->stream) - 1;
       if (timing) {
         CK(cudaEventRecord(c->events[c->ev_used].second, c->stream));
         c->ev_used++;
@@ -739,10 +739,20 @@ static bool passes_asked(const crash_run_opts& o) {
   return o.tile || o.seg_per_iter > 0 || o.resort_interval != 0 || o.pass_limit > 0;
 }
 
-// Form of the mixed transport of a step of `total` packets (the results do
-// not depend on it).
+// Packets from which the FP64 form sorts them into bundles.  Its walk costs a
+// warp about 600 FP64 instructions per crossing however few of its lanes walk:
+// in emission order the seven eighths of a corner source's packets that leave
+// at once leave their lanes idle, and in any grid the walks of a warp end
+// apart.  The sort (three launches, 20 us) is small against either from some
+// thousand packets on.
+constexpr int64_t kFp64Bundle = 8192;
+
+// Form of the transport of a step of `total` packets (the results do not
+// depend on it).
 static int transport_form(const crash_ctx* c, int64_t total) {
   const crash_run_opts& o = c->opts;
+  if (c->precision != CRASH_MIXED)
+    return total >= kFp64Bundle && c->n_src_total <= kMaxBundleKeys ? FORM_BUNDLE : FORM_DIRECT;
   if (!o.wavefront) return FORM_DIRECT;
   // (periodic boxes have no passes: their packets' path budget is not in a record)
   if (!c->any_periodic && passes_asked(o)) return FORM_PASSES;
@@ -810,7 +820,7 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
                      cudaMemcpyHostToDevice, c->stream));
   int form = FORM_DIRECT;
   bool per_launch = false;
-  if (c->precision == CRASH_MIXED) {
+  {
     // workspace: the packet queue (two record buffers) or the sort buffers
     // of the step's form, sized to the step (at most 2^28 packets per chunk:
     // 38 GB of queue with 8 bins, 3.2 GB of sort buffers); none when every
@@ -841,10 +851,17 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
       const size_t cap = memory_cap();
       const size_t need = (size_t)want.queue * (size_t)(2 * (((32 + 4 * c->n_bins) + 15) / 16 * 16)) +
                           12 * (size_t)std::max(want.queue, want.bundle) + 8 * (size_t)want.bundle_keys;
-      if (cap && c->bytes + need > cap)
-        return set_err(c, CRASH_ERR_OOM, "device memory cap (CRASH_DEVICE_MEMORY_CAP) exceeded by the packet workspace");
+      const bool fits = !cap || c->bytes + need <= cap;
+      if (!fits && form != FORM_BUNDLE)
+        return set_err(c, CRASH_ERR_OOM, "device memory cap (CRASH_DEVICE_MEMORY_CAP) exceeded by the packet queue");
       cudaError_t e = cudaSuccess;
-      c->wf = wavefront_create(want, c->n_bins, &e);
+      if (fits) c->wf = wavefront_create(want, c->n_bins, &e);
+      if (!c->wf && form == FORM_BUNDLE) {
+        // no room to sort: emission order needs none
+        cudaGetLastError();
+        form = FORM_DIRECT;
+        c->wf = wavefront_create(WFSize(), c->n_bins, &e);
+      }
       if (!c->wf) return set_err(c, CRASH_ERR_OOM, std::string("packet workspace: ") + cudaGetErrorString(e));
     }
   }

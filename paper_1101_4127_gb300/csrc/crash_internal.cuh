@@ -139,7 +139,9 @@ enum { ERR_DDA_LIMIT = 1, ERR_DIRECTION = 2, ERR_QUEUE = 4, ERR_WATCHDOG = 8 };
 // launchers implemented in the kernel translation units
 void launch_prep(const StepArgs& a, int precision, cudaStream_t s);
 void launch_budget(const StepArgs& a, const BinTables& t, cudaStream_t s);
-void launch_trace_fp64(const StepArgs& a, const BinTables& t, int block, cudaStream_t s);
+// wf: the workspace of the bundles' sort (a.form = FORM_BUNDLE); returns the
+// kernels launched
+int launch_trace_fp64(const StepArgs& a, const BinTables& t, int block, void* wf, cudaStream_t s);
 void launch_chemistry(const StepArgs& a, cudaStream_t s);
 // diffuse recombination field: pick this step's re-emitting cells (and
 // restart their counts), then trace one packet per cell in either form
@@ -179,5 +181,7 @@ void wavefront_destroy(void* w);
 WFSize wavefront_size(void* w);
 // the largest number of direction keys the bundle sort scans
 constexpr int64_t kMaxBundleKeys = (int64_t)4096 * 1024;
+// packet ids (from g0) of a chunk of n packets sorted by source and direction
+const unsigned* bundle_order(const StepArgs& a, void* wf, int64_t g0, int64_t n, cudaStream_t s);
 // threads the direct form keeps resident on the whole GPU
 int64_t resident_packets();

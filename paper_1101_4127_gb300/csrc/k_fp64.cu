@@ -213,15 +213,22 @@ __device__ __forceinline__ void walk_fp64(const StepArgs& a, const BinTables& t,
 #pragma unroll
       for (int j = 0; j < (NBT > 0 ? NBT : CRASH_MAX_BINS); ++j) {
         if (NBT == 0 && j >= nb) break;
+        // (an empty bin, and a species whose threshold lies above the bin, add
+        // exact zeros: left out)
+        const long long Nj = N[j];
+        if (Nj == 0) continue;
         const double kHI = nHI * t.sigma[0][j];
         double kap = kHI, kHeI = 0.0, kHeII = 0.0;
-        if (HE) {
+        const bool he1 = HE && t.sigma[1][j] > 0.0, he2 = HE && t.sigma[2][j] > 0.0;
+        if (he1) {
           kHeI = nHeI * t.sigma[1][j];
+          kap = kap + kHeI;
+        }
+        if (he2) {
           kHeII = nHeII * t.sigma[2][j];
-          kap = (kHI + kHeI) + kHeII;
+          kap = kap + kHeII;
         }
         const double f = exp_neg_spec(l * kap);
-        const long long Nj = N[j];
         long long Np = llrint((double)Nj * f);
         Np = Np > Nj ? Nj : Np;
         const long long A = Nj - Np;
@@ -229,22 +236,28 @@ __device__ __forceinline__ void walk_fp64(const StepArgs& a, const BinTables& t,
         left |= Np;
         if (A > 0) {
           long long A1 = 0, A2 = 0;
-          if (HE) {
-            A1 = llrint((double)A * (kHeI / kap));
-            A1 = A1 > A ? A : A1;
-            A2 = llrint((double)A * (kHeII / kap));
-            A2 = A2 > A - A1 ? A - A1 : A2;
+          const double Ad = (double)A;
+          if (he1 || he2) {
+            // both shares over the one kappa
+            const Divisor D(kap);
+            if (he1) {
+              A1 = llrint(Ad * D.of(kHeI));
+              A1 = A1 > A ? A : A1;
+            }
+            if (he2) {
+              A2 = llrint(Ad * D.of(kHeII));
+              A2 = A2 > A - A1 ? A - A1 : A2;
+            }
           }
           const long long A0 = A - A1 - A2;
           dHI += A0;
           dHeI += A1;
           dHeII += A2;
           if (HEAT) {
-            if (HE)
-              heat += ((double)A0 * t.wheat[0][j] + (double)A1 * t.wheat[1][j]) +
-                      (double)A2 * t.wheat[2][j];
-            else
-              heat += (double)A0 * t.wheat[0][j];
+            double w = (double)A0 * t.wheat[0][j];
+            if (he1) w = w + (double)A1 * t.wheat[1][j];
+            if (he2) w = w + (double)A2 * t.wheat[2][j];
+            heat += w;
           }
         }
       }
@@ -284,12 +297,14 @@ __device__ __forceinline__ void walk_fp64(const StepArgs& a, const BinTables& t,
 }
 
 template <int NBT, bool HE, bool HEAT>
-__global__ void __launch_bounds__(256) k_trace_fp64(StepArgs a, BinTables t) {
+__global__ void __launch_bounds__(256) k_trace_fp64(StepArgs a, BinTables t, const unsigned* order, int64_t g0,
+                                                    int64_t n) {
   const int nb = NBT > 0 ? NBT : t.n_bins;
-  const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t at = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   Tally tl{0, 0, 0, 0, 0};
   int b = -1;
-  if (gid < a.total_packets) {
+  if (at < n) {
+    const int64_t gid = g0 + (order ? (int64_t)__ldg(order + at) : at);
     b = box_of_packet(a.boxes, a.n_boxes, gid);
     const BoxMeta* M = a.boxes + b;
     const int64_t local = gid - M->pkt_off;
@@ -460,25 +475,33 @@ void launch_rec_fp64(const StepArgs& a, const BinTables& t, cudaStream_t s) {
 }
 
 template <int NBT, bool HE, bool HEAT>
-static void launch_t(const StepArgs& a, const BinTables& t, int block, cudaStream_t s) {
-  int64_t blocks = (a.total_packets + block - 1) / block;
-  k_trace_fp64<NBT, HE, HEAT><<<(unsigned)blocks, block, 0, s>>>(a, t);
+static int launch_t(const StepArgs& a, const BinTables& t, int block, void* wf, cudaStream_t s) {
+  int launches = 0;
+  const int64_t chunk = a.form == FORM_BUNDLE ? wavefront_size(wf).bundle : a.total_packets;
+  for (int64_t g0 = 0; g0 < a.total_packets; g0 += chunk) {
+    const int64_t n = std::min<int64_t>(chunk, a.total_packets - g0);
+    const unsigned* order = nullptr;
+    if (a.form == FORM_BUNDLE) {
+      order = bundle_order(a, wf, g0, n, s);
+      launches += 3;
+    }
+    k_trace_fp64<NBT, HE, HEAT><<<(unsigned)((n + block - 1) / block), block, 0, s>>>(a, t, order, g0, n);
+    ++launches;
+  }
+  return launches;
 }
 
-void launch_trace_fp64(const StepArgs& a, const BinTables& t, int block, cudaStream_t s) {
-  if (a.total_packets <= 0) return;
+int launch_trace_fp64(const StepArgs& a, const BinTables& t, int block, void* wf, cudaStream_t s) {
+  if (a.total_packets <= 0) return 1;
   if (block <= 0) block = 128;
   // the H+He kernels are exact for pure-H boxes too (their He terms are
   // +0), and isothermal boxes skip the heating deposit at run time
   const bool he = a.any_he != 0, heat = a.any_heat != 0;
-  if (t.n_bins == 1) {
-    if (he) { if (heat) launch_t<1, true, true>(a, t, block, s); else launch_t<1, true, false>(a, t, block, s); }
-    else { if (heat) launch_t<1, false, true>(a, t, block, s); else launch_t<1, false, false>(a, t, block, s); }
-  } else if (t.n_bins == 8) {
-    if (he) { if (heat) launch_t<8, true, true>(a, t, block, s); else launch_t<8, true, false>(a, t, block, s); }
-    else { if (heat) launch_t<8, false, true>(a, t, block, s); else launch_t<8, false, false>(a, t, block, s); }
-  } else {
-    if (he) { if (heat) launch_t<0, true, true>(a, t, block, s); else launch_t<0, true, false>(a, t, block, s); }
-    else { if (heat) launch_t<0, false, true>(a, t, block, s); else launch_t<0, false, false>(a, t, block, s); }
-  }
+#define CRASH_TRACE(NBT)                                                                                       \
+  (he ? (heat ? launch_t<NBT, true, true>(a, t, block, wf, s) : launch_t<NBT, true, false>(a, t, block, wf, s)) \
+      : (heat ? launch_t<NBT, false, true>(a, t, block, wf, s) : launch_t<NBT, false, false>(a, t, block, wf, s)))
+  if (t.n_bins == 1) return CRASH_TRACE(1);
+  if (t.n_bins == 8) return CRASH_TRACE(8);
+  return CRASH_TRACE(0);
+#undef CRASH_TRACE
 }

@@ -1591,6 +1591,24 @@ int source_of_packet(const StepArgs& a, int64_t gid) {
   return M->src_off + (int)((gid - M->pkt_off) / (M->win_hi - M->win_lo));
 }
 
+// Sort the n packets from g0 on by source and direction into wf->perm (three
+// launches); also clears the chunk's work counter.
+void sort_bundles(const StepArgs& a, const WF* wf, int64_t g0, int64_t n, cudaStream_t s) {
+  // the chunk's sources, each with 4^bits direction cells: about two packets
+  // to a cell, so that the 32 packets of a warp are neighbours
+  const int s0 = source_of_packet(a, g0);
+  const int64_t ns = source_of_packet(a, g0 + n - 1) - s0 + 1;
+  int bits = 0;
+  while (bits < 11 && (ns << (2 * bits + 2)) <= std::min<int64_t>(wf->bkeys, n / 2)) ++bits;
+  const int64_t nk = ns << (2 * bits);
+  cudaMemsetAsync(wf->count, 0, 4 * sizeof(unsigned), s);
+  cudaMemsetAsync(wf->bcount, 0, sizeof(unsigned) * nk, s);
+  const unsigned nsort = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 16);
+  k_bundle_count<<<nsort, 256, 0, s>>>(a, wf->key, wf->rank, wf->bcount, g0, n, s0, bits);
+  k_bundle_scan<<<(unsigned)((nk + 4095) / 4096), 1024, 0, s>>>(wf->bcount, wf->boff, wf->bsum, wf->count + 3, nk);
+  k_bundle_place<<<nsort, 256, 0, s>>>(wf->key, wf->rank, wf->boff, wf->bsum, wf->perm, n);
+}
+
 template <int NBT, bool HE, bool HEAT>
 int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF* wf, int max_iter,
               cudaStream_t s, EventPairs* ev, int* ev_used) {
@@ -1634,21 +1652,9 @@ int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF
   if (a.form == FORM_BUNDLE) {
     for (int64_t g0 = 0; g0 < a.total_packets; g0 += wf->bcap) {
       const int64_t n = std::min<int64_t>(wf->bcap, a.total_packets - g0);
-      // the chunk's sources, each with 4^bits direction cells: about two
-      // packets to a cell, so that the 32 packets of a warp are neighbours
-      const int s0 = source_of_packet(a, g0);
-      const int64_t ns = source_of_packet(a, g0 + n - 1) - s0 + 1;
-      int bits = 0;
-      while (bits < 11 && (ns << (2 * bits + 2)) <= std::min<int64_t>(wf->bkeys, n / 2)) ++bits;
-      const int64_t nk = ns << (2 * bits);
       WFArgs w = wf_args(wf, 0, true, false);
       w.work = wf->count + 2;
-      cudaMemsetAsync(wf->count, 0, 4 * sizeof(unsigned), s);
-      cudaMemsetAsync(wf->bcount, 0, sizeof(unsigned) * nk, s);
-      const unsigned nsort = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 16);
-      k_bundle_count<<<nsort, 256, 0, s>>>(a, wf->key, wf->rank, wf->bcount, g0, n, s0, bits);
-      k_bundle_scan<<<(unsigned)((nk + 4095) / 4096), 1024, 0, s>>>(wf->bcount, wf->boff, wf->bsum, wf->count + 3, nk);
-      k_bundle_place<<<nsort, 256, 0, s>>>(wf->key, wf->rank, wf->boff, wf->bsum, wf->perm, n);
+      sort_bundles(a, wf, g0, n, s);
       const unsigned ntrace = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 4);
       tic();
       if (a.any_periodic) k_trace_bundle<NBT, HE, HEAT, true><<<ntrace, 256, 0, s>>>(a, t, w, g0, n, max_iter);
@@ -1808,6 +1814,11 @@ int launch_trace_mixed(const StepArgs& a, const BinTables& t, const crash_run_op
   }
   if (cudaGetLastError() != cudaSuccess) return -1;
   return r;
+}
+
+const unsigned* bundle_order(const StepArgs& a, void* wf, int64_t g0, int64_t n, cudaStream_t s) {
+  sort_bundles(a, (const WF*)wf, g0, n, s);
+  return ((const WF*)wf)->perm;
 }
 
 int64_t resident_packets() { return (int64_t)num_sms() * 3 * 256; }

@@ -2,14 +2,15 @@
 order, sorted into bundles by source and direction, or in passes, at the
 sizes where the forms' rules and remainders lie (one thread's worth above the
 resident packets, partial warps and chunks, one source or many, each number
-of colours and each set of deposited values, periodic walks, batches)."""
+of colours and each set of deposited values, periodic walks, batches); the
+FP64 form's bundles equal the oracle."""
 import ctypes as C
 
 import numpy as np
 import pytest
 
 from paper_1101_4127_gb300 import inputs, native
-from _common import small_hhe_box
+from _common import assert_deposits_equal, pair, small_hhe_box
 
 pytestmark = pytest.mark.gpu
 FIELDS = [native.F_DEP_HI, native.F_DEP_HEI, native.F_DEP_HEII, native.F_DEP_E, native.F_BUDGET]
@@ -135,3 +136,36 @@ def test_noalloc_bundles_equal_emission_order(per_src):
         assert np.array_equal(h.read(f_).reshape(-1), got[:, k]), f_
     assert np.array_equal(h.read(native.F_BUDGET)[:5], budget[:5])
     h.close()
+
+
+@pytest.mark.parametrize("dims,n_src,per_src,bins,he,thin,opts", [
+    ((14, 11, 9), 1, 8191, 8, 0.08, False, {}),          # below the bundles' rule, and at it
+    ((14, 11, 9), 1, 8192, 8, 0.08, False, {}),
+    ((14, 11, 9), 3, 4001, 8, 0.08, True, dict(chunk_packets=3001)),
+    ((12, 12, 12), 2, 5003, 1, 0.0, False, {}),
+    ((12, 9, 7), 2, 4500, 5, 0.08, False, dict(pkt_begin=17)),
+])
+def test_fp64_bundles_equal_the_oracle(dims, n_src, per_src, bins, he, thin, opts):
+    box = small_hhe_box(dims, n_src=n_src, seed=760 + n_src, nbins=1 if bins == 1 else 8, thin=thin)
+    if bins not in (1, 8):
+        E, f = inputs.blackbody_bins(1e5, np.geomspace(13.6, 200.0, bins + 1))
+        box.bin_eV, box.bin_frac = E, np.tile(f, (n_src, 1))
+    box.he_over_h = he
+    g, o = pair(box)
+    g.set_options(chemistry=0, **opts)
+    o.set_options(chemistry=0, **{k: v for k, v in opts.items() if k != "chunk_packets"})
+    for _ in range(2):
+        g.step(DT, n_src * per_src)
+        o.step(DT, n_src * per_src)
+        assert_deposits_equal(g, o)
+    g.close()
+
+
+def test_fp64_step_without_room_to_sort_runs(monkeypatch):
+    box = small_hhe_box((10, 10, 10), n_src=1, seed=770)
+    monkeypatch.setenv("CRASH_DEVICE_MEMORY_CAP", str(250000))     # the grid's 150 kB, not 20000 packets' sort
+    g, o = pair(box)
+    g.step(DT, 20000)
+    o.step(DT, 20000)
+    assert_deposits_equal(g, o)
+    g.close()
