@@ -174,6 +174,75 @@ struct CellIn {
   bool helium;
 };
 
+// Bounds of the rates of change over a sub-step, in FP32: the sums of the
+// terms' sizes, which no rounding or cancellation exceeds.  A limit on the step
+// that cannot act even at the whole time left leaves the step as it is, so its
+// FP64 rates need not be formed (about 30 FP64 instructions for the fractions,
+// 70 for the temperature; a cell's last sub-step, often its only one, mostly
+// needs neither).  Values too small for FP32 count as 0 (of a rate per second,
+// 1e-38), too large or NaN ones as limits that may act.
+struct StepBound {
+  bool fractions, temperature;
+  float dT, room;           // |dT/dt| at most, and 0.999 eps T
+  __device__ __forceinline__ bool temperature_within(double h) const;
+};
+// v rounded towards 0 to FP32, on the integer unit (v >= 0)
+__device__ __forceinline__ float low(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), e = hi >> 20;
+  if (e - 897u >= 254u) return e < 897u ? 0.f : INFINITY;          // (negative numbers too: limits that may act)
+  return __uint_as_float(((e - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | ((unsigned)__double2loint(v) >> 29));
+}
+__device__ __forceinline__ bool StepBound::temperature_within(double h) const {
+  return temperature && !(dT * (low(h) * 1.001f) < room);
+}
+template <bool ISO>
+__device__ __forceinline__ StepBound step_bound(const CellIn& c, const Rates& r, double x, double y1, double y2,
+                                                double y3, double ne, double ntot, double T, double rem) {
+  StepBound q;
+  const double u = 1.0 - x;
+  q.fractions = true;
+  q.temperature = !ISO && !c.iso;
+  q.dT = INFINITY;
+  q.room = 0.f;
+  // (constant sources, fractions out of bounds: not bounded here)
+  if (nonzero(c.SH) || nonzero(c.S1) || nonzero(c.S2) || nonzero(c.heat_rate) || negative(x) || negative(u) ||
+      negative(y1) || negative(y2) || negative(y3))
+    return q;
+  const float X = low(x), U = low(u), E = low(ne), m = low(rem) * 1.001f, eps = low(c.eps) * 0.999f;
+  const float dx = (low(c.GH) + low(r.bHI) * E) * U + low(r.aHII) * E * X;
+  const float tiny = 1e-3f;
+  bool act = !(dx * m < eps * fminf(fmaxf(U, tiny), fmaxf(X, tiny)));
+  float Y1 = 0.f, Y2 = 0.f, Y3 = 0.f, dy1 = 0.f, dy3 = 0.f;
+  if (c.helium) {
+    Y1 = low(y1);
+    Y2 = low(y2);
+    Y3 = low(y3);
+    dy1 = (low(c.G1) + low(r.bHeI) * E) * Y1 + (low(r.aHeII) + low(r.adiel)) * E * Y2;
+    dy3 = (low(c.G2) + low(r.bHeII) * E) * Y2 + low(r.aHeIII) * E * Y3;
+    act = act || !(dy1 * m < eps * fmaxf(Y1, tiny) && (dy1 + dy3) * m < eps * fmaxf(Y2, tiny) &&
+                   dy3 * m < eps * fmaxf(Y3, tiny));
+  }
+  q.fractions = act;
+  if (!ISO && !c.iso) {
+    const float k = (float)(1.0 / (1.5 * kB)), nH = low(c.nH), nHe = low(c.nHe), t = low(T);
+    // per second and cm^3, over 1.5 k: heating, cooling per electron
+    const float heat = (low(c.WH) * k) * (nH * U) + ((low(c.W1) * k) * (nHe * Y1) + (low(c.W2) * k) * (nHe * Y2));
+    const float ff = low(r.cff) * k;
+    const float H1 = (low(r.cexHI) + low(r.cionHI)) * k, H2 = low(r.crecHII) * k + ff;
+    float cool = H1 * (nH * U) + H2 * (nH * X);
+    if (c.helium) {
+      const float He2 = ((low(r.cexHeII) + low(r.cionHeII)) + (low(r.crecHeII) + low(r.cdiel))) * k + ff;
+      cool += (low(r.cionHeI) * k) * (nHe * Y1) + He2 * (nHe * Y2) + (low(r.crecHeIII) * k + 4.f * ff) * (nHe * Y3);
+    }
+    cool += (low(c.ccomp) * k) * (t + low(c.Tcmb));
+    const float dne = nH * dx + nHe * (dy1 + 3.f * dy3);
+    q.dT = ((heat + cool * E) + t * dne) * 1.001f / low(ntot);
+    q.room = eps * t;
+    q.temperature = !(q.dT * m < q.room);
+  }
+  return q;
+}
+
 // One sub-step of the cell integration; updates x (HII), y2 (HeII), y3
 // (HeIII), T and the remaining time rem (0 after the last sub-step).  COUNT
 // (diffuse recombination field): adds to nrec[] the recombinations straight
@@ -206,42 +275,46 @@ __device__ __forceinline__ void substep(const CellIn& c, Rates& r, Rates& rB, do
   const double y1 = (1.0 - y2) - y3;
   const double ne = c.nH * x + c.nHe * (y2 + 2.0 * y3);
   const double GH = c.GH, G1 = c.G1, G2 = c.G2;
-  // rates of change at the start of the sub-step (for the step size)
-  const double IH = GH + bH * ne, RH = aH * ne;
-  const double I1 = G1 + bHe1 * ne, R2 = aHe2 * ne, I2 = G2 + bHe2 * ne, R3 = aHe3 * ne;
-  // constant sources (photon-conserving coupling), for the step size at most
-  // what the atoms present can take over the time left.  With no source
-  // (the default coupling) and a fraction that is not negative the cap is
-  // min(0, v >= 0) = 0: the FP64 division is skipped, the value is the same
-  double sH = (nonzero(c.SH) || negative(1.0 - x)) ? fmin(c.SH, quotient(1.0 - x, rem)) : 0.0;
-  double s1 = (nonzero(c.S1) || negative(y1)) ? fmin(c.S1, quotient(y1, rem)) : 0.0;
-  double s2 = (nonzero(c.S2) || negative(y2)) ? fmin(c.S2, quotient(y2, rem)) : 0.0;
-  const double dx = (sH + IH * (1.0 - x)) - RH * x;
-  const double dy1 = (-I1 * y1 + R2 * y2) - s1;
-  const double dy3 = (s2 + I2 * y2) - R3 * y3;
-  const double dy2 = -dy1 - dy3;
-  double h = rem;
-  {
-    const double val[5] = {1.0 - x, x, y1, y2, y3};
-    const double der[5] = {-dx, dx, dy1, dy2, dy3};
-    const int nv = he ? 5 : 2;
-    for (int i = 0; i < nv; ++i) {
-      const double fl = above(val[i], 1e-3) ? val[i] : 1e-3;
-      const double ad = fabs(der[i]);
-      if (above(ad * h, c.eps * fl)) h = quotient(c.eps * fl, ad);
-    }
-  }
+  double h = rem, sH, s1, s2;
   const double ntot = c.nH + c.nHe + ne;
-  if (!ISO && !c.iso) {
-    const double nHI = c.nH * (1.0 - x), nHII = c.nH * x;
-    const double heat = (c.WH * nHI + c.W1 * (c.nHe * y1) + c.W2 * (c.nHe * y2)) + c.heat_rate;
-    const double L = cooling_rate(r, c.mask, ne, nHI, nHII, c.nHe * y1, c.nHe * y2, c.nHe * y3) +
-                     c.ccomp * ne * (T - c.Tcmb);
-    const double dne = c.nH * dx + c.nHe * (dy2 + 2.0 * dy3);
-    // (dT is only the step-size estimate: the reciprocal constant's rounding does not matter)
-    const double dT = quotient((heat - L) * (1.0 / (1.5 * kB)) - T * dne, ntot);
-    const double adT = fabs(dT);
-    if (above(adT * h, c.eps * T)) h = quotient(c.eps * T, adT);
+  // which limits on the step can act at all, from bounds in FP32
+  const StepBound q = step_bound<ISO>(c, r, x, y1, y2, y3, ne, ntot, T, rem);
+  if (q.fractions || q.temperature) {
+    // rates of change at the start of the sub-step (for the step size)
+    const double IH = GH + bH * ne, RH = aH * ne;
+    const double I1 = G1 + bHe1 * ne, R2 = aHe2 * ne, I2 = G2 + bHe2 * ne, R3 = aHe3 * ne;
+    // constant sources (photon-conserving coupling), for the step size at most
+    // what the atoms present can take over the time left.  With no source
+    // (the default coupling) and a fraction that is not negative the cap is
+    // min(0, v >= 0) = 0: the FP64 division is skipped, the value is the same
+    sH = (nonzero(c.SH) || negative(1.0 - x)) ? fmin(c.SH, quotient(1.0 - x, rem)) : 0.0;
+    s1 = (nonzero(c.S1) || negative(y1)) ? fmin(c.S1, quotient(y1, rem)) : 0.0;
+    s2 = (nonzero(c.S2) || negative(y2)) ? fmin(c.S2, quotient(y2, rem)) : 0.0;
+    const double dx = (sH + IH * (1.0 - x)) - RH * x;
+    const double dy1 = (-I1 * y1 + R2 * y2) - s1;
+    const double dy3 = (s2 + I2 * y2) - R3 * y3;
+    const double dy2 = -dy1 - dy3;
+    if (q.fractions) {
+      const double val[5] = {1.0 - x, x, y1, y2, y3};
+      const double der[5] = {-dx, dx, dy1, dy2, dy3};
+      const int nv = he ? 5 : 2;
+      for (int i = 0; i < nv; ++i) {
+        const double fl = above(val[i], 1e-3) ? val[i] : 1e-3;
+        const double ad = fabs(der[i]);
+        if (above(ad * h, c.eps * fl)) h = quotient(c.eps * fl, ad);
+      }
+    }
+    if (!ISO && !c.iso && q.temperature_within(h)) {
+      const double nHI = c.nH * (1.0 - x), nHII = c.nH * x;
+      const double heat = (c.WH * nHI + c.W1 * (c.nHe * y1) + c.W2 * (c.nHe * y2)) + c.heat_rate;
+      const double L = cooling_rate(r, c.mask, ne, nHI, nHII, c.nHe * y1, c.nHe * y2, c.nHe * y3) +
+                       c.ccomp * ne * (T - c.Tcmb);
+      const double dne = c.nH * dx + c.nHe * (dy2 + 2.0 * dy3);
+      // (dT is only the step-size estimate: the reciprocal constant's rounding does not matter)
+      const double dT = quotient((heat - L) * (1.0 / (1.5 * kB)) - T * dne, ntot);
+      const double adT = fabs(dT);
+      if (above(adT * h, c.eps * T)) h = quotient(c.eps * T, adT);
+    }
   }
   if (nsub == c.max_sub - 1 || !above(rem, h)) h = rem;
   // the sources of the sub-step ionise at most the atoms present (He II also
