@@ -434,6 +434,12 @@ void cross_sections(int nb, const double* E, BinTables& t, int& heatF) {
     t.sigma32_max[s] = 0.f;
     for (int j = 0; j < nb; ++j) t.sigma32_max[s] = std::max(t.sigma32_max[s], t.sigma32[s][j]);
   }
+  for (int j = 0; j < CRASH_MAX_BINS; j += 2) {
+    auto at = [&](const float* v, int k) { return k < nb ? v[k] : 0.f; };
+    const float* s[6] = {t.sigma32[0], t.sigma32[1], t.sigma32[2], t.sw32[0], t.sw32[1], t.sw32[2]};
+    for (int k = 0; k < 3; ++k)
+      t.pairs[k][j / 2] = make_float4(at(s[2 * k], j), at(s[2 * k], j + 1), at(s[2 * k + 1], j), at(s[2 * k + 1], j + 1));
+  }
   t.n_bins = nb;
 }
 

@@ -73,6 +73,8 @@ struct BinTables {
   float wheat32[3][CRASH_MAX_BINS];
   float sigma32_max[3];              // largest sigma32 of each species over the bins
   float sw32[3][CRASH_MAX_BINS];     // sigma32 * wheat32 (FP32 product): heating weight per unit t_s
+  // sigma32 and sw32 by bin pairs, as 16-byte loads: (H I, He I), (He II, sw H I), (sw He I, sw He II)
+  float4 pairs[3][CRASH_MAX_BINS / 2];
 };
 
 // Forms of the mixed transport (chosen per step by transport_form):

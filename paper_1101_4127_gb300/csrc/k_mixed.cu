@@ -146,9 +146,9 @@ __device__ __forceinline__ long long float_to_ll(float x) {
 // rint of the three per-cell shares x1, x2, xh (each at most about the
 // cell's absorbed total Au): with Au below 2^31 all three fit the 32-bit
 // conversion, which is then the whole rounding
-__device__ __forceinline__ void round_shares(long long Au, float x1, float x2, float xh, long long& a1,
-                                             long long& a2, long long& h) {
-  if ((unsigned long long)Au < 0x80000000ull) {
+__device__ __forceinline__ void round_shares(const unsigned lanes, long long Au, float x1, float x2, float xh,
+                                             long long& a1, long long& a2, long long& h) {
+  if (!__any_sync(lanes, (unsigned long long)Au >= 0x80000000ull)) {
     a1 = (long long)__float2uint_rn(x1);
     a2 = (long long)__float2uint_rn(x2);
     h = (long long)__float2uint_rn(xh);
@@ -274,12 +274,13 @@ __device__ __forceinline__ unsigned absorb_thick(unsigned m, float Nf, float tau
 // some bin may have tau >= 0.5 (known from one bound for the whole cell): no
 // bin is looked at on its own, and the packet's liveness is unchanged (left
 // is not recomputed).  Otherwise every bin pair is done by the series first
-// and its bins with tau >= 0.5, if any lane has some, are done again, so that
-// lanes in thin and in thick cells share one instruction stream; and a pair
-// that holds no photons in any lane (soft bins die within the first thick
+// and, if any lane has a thick bin in it, both ways, each lane taking its own,
+// so that lanes in thin and in thick cells share one instruction stream; and a
+// pair that holds no photons in any lane (soft bins die within the first thick
 // cells) is left out: it absorbs nothing and adds nothing.
+// lanes: the lanes that call together.
 template <int NBT, bool HE, bool HEAT, bool THIN>
-__device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 tHeI2, const f32x2 tHeII2,
+__device__ __forceinline__ void attenuate_bins_x2(const unsigned lanes, const f32x2 tHI2, const f32x2 tHeI2, const f32x2 tHeII2,
                                                   Content<NBT>& c, const BinTables& t,
                                                   unsigned long long& At, unsigned& left, f32x2& g1,
                                                   f32x2& g2, f32x2& h0, f32x2& h1, f32x2& h2) {
@@ -287,13 +288,14 @@ __device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 
 #pragma unroll
   for (int j = 0; j < NBT; j += 2) {
     const unsigned m0 = c.m[j], m1 = c.m[j + 1];
-    if (!THIN && (m0 | m1) == 0u) continue;
-    const f32x2 s0 = f2(t.sigma32[0][j], t.sigma32[0][j + 1]);
+    if (!THIN && !__any_sync(lanes, (m0 | m1) != 0u)) continue;
+    const float4 t01 = t.pairs[0][j / 2], t23 = t.pairs[1][j / 2], t45 = t.pairs[2][j / 2];
+    const f32x2 s0 = f2(t01.x, t01.y);
     f32x2 tau = f2_mul(tHI2, s0);
     f32x2 s1 = 0ull, s2 = 0ull;
     if (HE) {
-      s1 = f2(t.sigma32[1][j], t.sigma32[1][j + 1]);
-      s2 = f2(t.sigma32[2][j], t.sigma32[2][j + 1]);
+      s1 = f2(t01.z, t01.w);
+      s2 = f2(t23.x, t23.y);
       tau = f2_fma(tHeII2, s2, f2_fma(tHeI2, s1, tau));
     }
     const float N0 = __uint2float_rn(m0), N1 = __uint2float_rn(m1);
@@ -313,12 +315,15 @@ __device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 
     if (!THIN) {
       float tau0, tau1;
       f2_split(tau, tau0, tau1);
-      if (fmaxf(tau0, tau1) >= 0.5f) {
-        float q0, q1;
+      // (not below 0.5: NaN, an infinite opacity times 0, absorbs everything)
+      const bool thick0 = !(tau0 < 0.5f), thick1 = !(tau1 < 0.5f);
+      if (__any_sync(lanes, thick0 || thick1)) {
+        float q0, q1, p0, p1;
         f2_split(q2, q0, q1);
-        if (tau0 >= 0.5f) A0 = absorb_thick(m0, N0, tau0, q0);
-        if (tau1 >= 0.5f) A1 = absorb_thick(m1, N1, tau1, q1);
-        q2 = f2(q0, q1);
+        const unsigned B0 = absorb_thick(m0, N0, tau0, p0), B1 = absorb_thick(m1, N1, tau1, p1);
+        A0 = thick0 ? B0 : A0;
+        A1 = thick1 ? B1 : A1;
+        q2 = f2(thick0 ? p0 : q0, thick1 ? p1 : q1);
       }
     }
     c.m[j] = m0 - A0;
@@ -330,10 +335,10 @@ __device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 
       g2 = f2_fma(q2, s2, g2);
     }
     if (HEAT) {
-      h0 = f2_fma(q2, f2(t.sw32[0][j], t.sw32[0][j + 1]), h0);
+      h0 = f2_fma(q2, f2(t23.z, t23.w), h0);
       if (HE) {
-        h1 = f2_fma(q2, f2(t.sw32[1][j], t.sw32[1][j + 1]), h1);
-        h2 = f2_fma(q2, f2(t.sw32[2][j], t.sw32[2][j + 1]), h2);
+        h1 = f2_fma(q2, f2(t45.x, t45.y), h1);
+        h2 = f2_fma(q2, f2(t45.z, t45.w), h2);
       }
     }
   }
@@ -350,7 +355,7 @@ __device__ __forceinline__ float f2_sum(f32x2 v) {
 // the packet's units), scaled to photon quanta and rounded once: He I and
 // He II clamped to the absorbed total, H I taking the rest.
 template <bool HE, bool HEAT>
-__device__ __forceinline__ void cell_shares(unsigned long long At, int e, float tHI, float tHeI, float tHeII,
+__device__ __forceinline__ void cell_shares(const unsigned lanes, unsigned long long At, int e, float tHI, float tHeI, float tHeII,
                                             float G1, float G2, float H0, float H1, float H2,
                                             long long& dHI, long long& dHeI, long long& dHeII,
                                             long long& dE) {
@@ -360,12 +365,12 @@ __device__ __forceinline__ void cell_shares(unsigned long long At, int e, float 
   const float fHeI = HE ? tHeI * G1 : 0.f, fHeII = HE ? tHeII * G2 : 0.f;
   const float fheat = HEAT ? (HE ? fmaf(tHeII, H2, fmaf(tHeI, H1, tHI * H0)) : tHI * H0) : 0.f;
   long long a1, a2, h;
-  round_shares(Au, fHeI * unit, fHeII * unit, fheat * unit, a1, a2, h);
+  round_shares(lanes, Au, fHeI * unit, fHeII * unit, fheat * unit, a1, a2, h);
   if (!HE) a1 = a2 = 0;
   if (!HEAT) h = 0;
   // He shares above the cell's total only by rounding: clamp then (the
   // clamps change nothing when the two fit)
-  if (HE && (unsigned long long)a1 + (unsigned long long)a2 > (unsigned long long)Au) {
+  if (HE && __any_sync(lanes, (unsigned long long)a1 + (unsigned long long)a2 > (unsigned long long)Au)) {
     a1 = a1 > Au ? Au : a1;
     a2 = a2 > Au - a1 ? Au - a1 : a2;
   }
@@ -378,7 +383,7 @@ __device__ __forceinline__ void cell_shares(unsigned long long At, int e, float 
 // left: on entry, nonzero if some bin holds photons; on return, the same
 // after the cell
 template <int NBT, bool HE, bool HEAT>
-__device__ __forceinline__ long long cell_attenuate_x2(float seg, float dl, float4 ab, Content<NBT>& c,
+__device__ __forceinline__ long long cell_attenuate_x2(const unsigned lanes, float seg, float dl, float4 ab, Content<NBT>& c,
                                                        const BinTables& t, long long& dHI,
                                                        long long& dHeI, long long& dHeII, long long& dE,
                                                        unsigned& left) {
@@ -393,11 +398,11 @@ __device__ __forceinline__ long long cell_attenuate_x2(float seg, float dl, floa
   const float k0max = tHI * t.sigma32_max[0];
   const float tau_max = HE ? fmaf(tHeII, t.sigma32_max[2], fmaf(tHeI, t.sigma32_max[1], k0max)) : k0max;
   // (either form gives a lane in a thin cell the same bits: the vote only picks the instruction stream)
-  if (!__any_sync(__activemask(), !(tau_max < 0.5f)))
-    attenuate_bins_x2<NBT, HE, HEAT, true>(tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
+  if (!__any_sync(lanes, !(tau_max < 0.5f)))
+    attenuate_bins_x2<NBT, HE, HEAT, true>(lanes, tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
   else
-    attenuate_bins_x2<NBT, HE, HEAT, false>(tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
-  cell_shares<HE, HEAT>(At, c.e, tHI, tHeI, tHeII, f2_sum(g1), f2_sum(g2), f2_sum(h0), f2_sum(h1),
+    attenuate_bins_x2<NBT, HE, HEAT, false>(lanes, tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
+  cell_shares<HE, HEAT>(lanes, At, c.e, tHI, tHeI, tHeII, f2_sum(g1), f2_sum(g2), f2_sum(h0), f2_sum(h1),
                         f2_sum(h2), dHI, dHeI, dHeII, dE);
   return (long long)(At << c.e);
 }
@@ -409,12 +414,12 @@ __device__ __forceinline__ long long cell_attenuate_x2(float seg, float dl, floa
 // species and heating sums run over the even and the odd bins separately
 // and are then added, as the two lanes of the packed form do.
 template <int NBT, bool HE, bool HEAT>
-__device__ __forceinline__ long long cell_attenuate(float seg, float dl, float4 ab, Content<NBT>& c,
-                                                    int nb, const BinTables& t, long long& dHI,
+__device__ __forceinline__ long long cell_attenuate(const unsigned lanes, float seg, float dl, float4 ab,
+                                                    Content<NBT>& c, int nb, const BinTables& t, long long& dHI,
                                                     long long& dHeI, long long& dHeII, long long& dE,
                                                     unsigned& left) {
   if constexpr (NBT >= 2 && NBT % 2 == 0)
-    return cell_attenuate_x2<NBT, HE, HEAT>(seg, dl, ab, c, t, dHI, dHeI, dHeII, dE, left);
+    return cell_attenuate_x2<NBT, HE, HEAT>(lanes, seg, dl, ab, c, t, dHI, dHeI, dHeII, dE, left);
   const float l = seg * dl;
   const float tHI = l * ab.x, tHeI = l * ab.y, tHeII = l * ab.z;
   unsigned long long At = 0;
@@ -447,7 +452,7 @@ __device__ __forceinline__ long long cell_attenuate(float seg, float dl, float4 
     }
     left |= mj;
   }
-  cell_shares<HE, HEAT>(At, c.e, tHI, tHeI, tHeII, g1[0] + g1[1], g2[0] + g2[1], h0[0] + h0[1],
+  cell_shares<HE, HEAT>(lanes, At, c.e, tHI, tHeI, tHeII, g1[0] + g1[1], g2[0] + g2[1], h0[0] + h0[1],
                         h1[0] + h1[1], h2[0] + h2[1], dHI, dHeI, dHeII, dE);
   return (long long)(At << c.e);
 }
@@ -532,24 +537,20 @@ struct GlobalCells {
 #pragma unroll
     for (int q = 1; q < 4; ++q) {
       const unsigned long long v = *reinterpret_cast<const unsigned long long*>(src + 16 * q);
-      if (cq[q] == cur) {
-        acc += v;
-      } else {
-        if (cur != none && acc) atomicAdd(dk + 4 * (size_t)cur, acc);
-        cur = cq[q];
-        acc = v;
-        whole = false;
-      }
+      const bool other = cq[q] != cur;
+      if (other && cur != none && acc) atomicAdd(dk + 4 * (size_t)cur, acc);
+      acc = (other ? 0ull : acc) + v;
+      cur = cq[q];
+      whole = whole && !other;
     }
     if (__any_sync(0xFFFFFFFFu, whole)) {
 #pragma unroll
       for (int o = 4; o < 32; o <<= 1) {
         const unsigned other = __shfl_xor_sync(0xFFFFFFFFu, cur, o);
         const unsigned long long v = __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-        if (other == cur) {
-          if (lane & o) cur = none;
-          else acc += v;
-        }
+        const bool same = other == cur;
+        acc += same ? v : 0ull;             // (the upper lane's sum is not sent)
+        cur = same && (lane & o) ? none : cur;
       }
     }
     if (cur != none && acc) atomicAdd(dk + 4 * (size_t)cur, acc);
@@ -633,47 +634,52 @@ __device__ __forceinline__ int walk_steps(const bool run, int& ix, int& iy, int&
     next = cells.index(ix, iy, iz);
     ab = cells.load(next);
   }
+  // A lane that is done goes on with segments of no length, which absorb
+  // nothing, load nothing and are no crossings: the warp stays in one
+  // instruction stream, whose branches are votes of all lanes.  (Its step
+  // counts move on past the face it left through, or no longer matter.)
   for (int it = 1;; ++it) {
     if (Cells::kWarp ? !__any_sync(0xFFFFFFFFu, go) : !go) break;
+    const unsigned lanes = Cells::kWarp ? 0xFFFFFFFFu : __activemask();
     const unsigned cell = next;
-    bool has = false;
-    long long dHI = 0, dHeI = 0, dHeII = 0, dE = 0;
-    if (go) {
-      // step the walk into the next cell (ties x before y before z) and
-      // request its absorbers
-      float seg = fminf(tMx, fminf(tMy, tMz));
-      const bool bx = tMx == seg, by = !bx && tMy == seg, bz = !bx && !by;
-      tMx = bx ? tDx : tMx - seg;
-      tMy = by ? tDy : tMy - seg;
-      tMz = bz ? tDz : tMz - seg;
-      rx -= bx ? 1 : 0;
-      ry -= by ? 1 : 0;
-      rz -= bz ? 1 : 0;
-      next += bx ? stx : (by ? sty : stz);
-      bool leave = min(rx, min(ry, rz)) == 0;
-      if (PER && per && leave) {
-        // back in through the opposite face
-        if (rx == 0) { rx = R.x1 - R.x0; next -= stx * (unsigned)rx; }
-        if (ry == 0) { ry = R.y1 - R.y0; next -= sty * (unsigned)ry; }
-        if (rz == 0) { rz = R.z1 - R.z0; next -= stz * (unsigned)rz; }
-        leave = false;
-      }
-      const float4 here = ab;
-      if (!leave) ab = cells.load(next);
-      // periodic: the path left to the light-travel distance cuts the segment
-      if (PER && per) {
-        cut = seg >= *trem;
-        if (cut) seg = *trem;
-        *trem -= seg;
-      }
-      go = !(leave || it >= max_iter || (PER && cut));
-      // attenuate and deposit in the current cell (a segment of no length
-      // absorbs nothing and is no crossing)
-      has = cell_attenuate<NBT, HE, HEAT>(seg, dl, here, N, nb, t, dHI, dHeI, dHeII, dE, left) != 0;
-      tl.crossings += seg > 0.f ? 1u : 0u;
-      if (left == 0 && seg > 0.f) go = false;
-      if (!heat_box) dE = 0;
+    // step the walk into the next cell (ties x before y before z) and request
+    // its absorbers
+    float seg = fminf(tMx, fminf(tMy, tMz));
+    const bool bx = tMx == seg, by = !bx && tMy == seg, bz = !bx && !by;
+    tMx = bx ? tDx : tMx - seg;
+    tMy = by ? tDy : tMy - seg;
+    tMz = bz ? tDz : tMz - seg;
+    rx -= bx ? 1 : 0;
+    ry -= by ? 1 : 0;
+    rz -= bz ? 1 : 0;
+    next += bx ? stx : (by ? sty : stz);
+    bool leave = min(rx, min(ry, rz)) <= 0;
+    if (PER && per && leave) {
+      // back in through the opposite face
+      if (rx == 0) { rx = R.x1 - R.x0; next -= stx * (unsigned)rx; }
+      if (ry == 0) { ry = R.y1 - R.y0; next -= sty * (unsigned)ry; }
+      if (rz == 0) { rz = R.z1 - R.z0; next -= stz * (unsigned)rz; }
+      leave = false;
     }
+    const float4 here = ab;
+    const bool went = go;
+    if (went && !leave) ab = cells.load(next);
+    // periodic: the path left to the light-travel distance cuts the segment
+    if (PER && per && went) {
+      cut = seg >= *trem;
+      if (cut) seg = *trem;
+      *trem -= seg;
+    }
+    go = went && !(leave || it >= max_iter || (PER && cut));
+    seg = went ? seg : 0.f;
+    if (!go) ab = make_float4(0.f, 0.f, 0.f, 0.f);      // what a lane that is done crosses from now on
+    // attenuate and deposit in the current cell (a segment of no length
+    // absorbs nothing and is no crossing)
+    long long dHI, dHeI, dHeII, dE;
+    const bool has = cell_attenuate<NBT, HE, HEAT>(lanes, seg, dl, here, N, nb, t, dHI, dHeI, dHeII, dE, left) != 0;
+    tl.crossings += seg > 0.f ? 1u : 0u;
+    if (left == 0 && seg > 0.f) go = false;
+    if (!heat_box) dE = 0;
     cells.add(has, cell, dHI, dHeI, dHeII, dE);
   }
   ix = dx > 0.f ? R.x1 - rx : R.x0 + rx - 1;
