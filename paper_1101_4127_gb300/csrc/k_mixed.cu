@@ -137,26 +137,10 @@ __device__ __forceinline__ void flush_warp(const StepArgs& a, int b, Tally& t) {
 // conversions: hi = floor(x / 2^32) and the rest x - hi 2^32, which the fma
 // gives exactly (below 2^32 the rest is x itself; above it x is an integer
 // whose low part fits the 24-bit significand, or hi holds all of x).
-__device__ __forceinline__ long long float_to_ll(float x) {
+__device__ __forceinline__ unsigned long long float_to_ull(float x) {
   const unsigned hi = __float2uint_rz(x * 2.3283064365386963e-10f);
   const unsigned lo = __float2uint_rn(fmaf(-__uint2float_rn(hi), 4294967296.0f, x));
-  return (long long)(((unsigned long long)hi << 32) | lo);
-}
-
-// rint of the three per-cell shares x1, x2, xh (each at most about the
-// cell's absorbed total Au): with Au below 2^31 all three fit the 32-bit
-// conversion, which is then the whole rounding
-__device__ __forceinline__ void round_shares(const unsigned lanes, long long Au, float x1, float x2, float xh,
-                                             long long& a1, long long& a2, long long& h) {
-  if (!__any_sync(lanes, (unsigned long long)Au >= 0x80000000ull)) {
-    a1 = (long long)__float2uint_rn(x1);
-    a2 = (long long)__float2uint_rn(x2);
-    h = (long long)__float2uint_rn(xh);
-  } else {
-    a1 = float_to_ll(x1);
-    a2 = float_to_ll(x2);
-    h = float_to_ll(xh);
-  }
+  return ((unsigned long long)hi << 32) | lo;
 }
 
 // (1 - exp(-tau)) / tau for 0 <= tau <= 0.5: a degree-5 polynomial fitted
@@ -353,40 +337,48 @@ __device__ __forceinline__ float f2_sum(f32x2 v) {
 
 // The cell's species and heating shares from the per-species bin sums (in
 // the packet's units), scaled to photon quanta and rounded once: He I and
-// He II clamped to the absorbed total, H I taking the rest.
-template <bool HE, bool HEAT>
-__device__ __forceinline__ void cell_shares(const unsigned lanes, unsigned long long At, int e, float tHI, float tHeI, float tHeII,
-                                            float G1, float G2, float H0, float H1, float H2,
-                                            long long& dHI, long long& dHeI, long long& dHeII,
-                                            long long& dE) {
-  // (with At = 0 the caller sends nothing, whatever comes out here)
-  const long long Au = (long long)(At << e);
+// He II clamped to the absorbed total, H I taking the rest; and the crossing's
+// deposit of them in `cell`.  Each share is at most about the absorbed total:
+// while no lane absorbs 2^31 quanta the shares are 32-bit numbers, one
+// conversion each is the whole rounding, and the record is half as long.
+template <bool HE, bool HEAT, class Cells>
+__device__ __forceinline__ void deposit_shares(const unsigned lanes, unsigned long long At, int e, float tHI, float tHeI,
+                                               float tHeII, float G1, float G2, float H0, float H1, float H2,
+                                               const Cells& cells, unsigned cell, bool heat_box) {
+  const unsigned long long Au = At << e;
+  const bool has = Au != 0ull;         // (with none absorbed nothing is sent, whatever the sums say)
   const float unit = __uint_as_float((unsigned)(127 + e) << 23);
   const float fHeI = HE ? tHeI * G1 : 0.f, fHeII = HE ? tHeII * G2 : 0.f;
   const float fheat = HEAT ? (HE ? fmaf(tHeII, H2, fmaf(tHeI, H1, tHI * H0)) : tHI * H0) : 0.f;
-  long long a1, a2, h;
-  round_shares(lanes, Au, fHeI * unit, fHeII * unit, fheat * unit, a1, a2, h);
-  if (!HE) a1 = a2 = 0;
-  if (!HEAT) h = 0;
-  // He shares above the cell's total only by rounding: clamp then (the
-  // clamps change nothing when the two fit)
-  if (HE && __any_sync(lanes, (unsigned long long)a1 + (unsigned long long)a2 > (unsigned long long)Au)) {
-    a1 = a1 > Au ? Au : a1;
-    a2 = a2 > Au - a1 ? Au - a1 : a2;
+  const float x1 = fHeI * unit, x2 = fHeII * unit, xh = heat_box ? fheat * unit : 0.f;
+  if (!__any_sync(lanes, Au >= 0x80000000ull)) {
+    const unsigned A = (unsigned)Au;
+    unsigned a1 = HE ? __float2uint_rn(x1) : 0u, a2 = HE ? __float2uint_rn(x2) : 0u;
+    const unsigned h = HEAT ? __float2uint_rn(xh) : 0u;
+    // He shares above the cell's total only by rounding: clamp then (the
+    // clamps change nothing when the two fit; neither nears 2^32)
+    if (HE && __any_sync(lanes, (unsigned long long)a1 + a2 > A)) {
+      a1 = a1 > A ? A : a1;
+      a2 = a2 > A - a1 ? A - a1 : a2;
+    }
+    cells.add(has, cell, make_uint4(A - a1 - a2, a1, a2, h));
+  } else {
+    unsigned long long a1 = HE ? float_to_ull(x1) : 0ull, a2 = HE ? float_to_ull(x2) : 0ull;
+    const unsigned long long h = HEAT ? float_to_ull(xh) : 0ull;
+    if (HE && __any_sync(lanes, a1 + a2 > Au)) {
+      a1 = a1 > Au ? Au : a1;
+      a2 = a2 > Au - a1 ? Au - a1 : a2;
+    }
+    cells.add(has, cell, Au - a1 - a2, a1, a2, h);
   }
-  dHeI = a1;
-  dHeII = a2;
-  dHI = Au - a1 - a2;
-  dE = h;
 }
 
 // left: on entry, nonzero if some bin holds photons; on return, the same
 // after the cell
-template <int NBT, bool HE, bool HEAT>
-__device__ __forceinline__ long long cell_attenuate_x2(const unsigned lanes, float seg, float dl, float4 ab, Content<NBT>& c,
-                                                       const BinTables& t, long long& dHI,
-                                                       long long& dHeI, long long& dHeII, long long& dE,
-                                                       unsigned& left) {
+template <int NBT, bool HE, bool HEAT, class Cells>
+__device__ __forceinline__ void cell_attenuate_x2(const unsigned lanes, float seg, float dl, float4 ab, Content<NBT>& c,
+                                                  const BinTables& t, unsigned& left, const Cells& cells,
+                                                  unsigned cell, bool heat_box) {
   static_assert(NBT >= 2 && NBT % 2 == 0, "bin pairs");
   const float l = seg * dl;
   const float tHI = l * ab.x, tHeI = l * ab.y, tHeII = l * ab.z;
@@ -402,24 +394,21 @@ __device__ __forceinline__ long long cell_attenuate_x2(const unsigned lanes, flo
     attenuate_bins_x2<NBT, HE, HEAT, true>(lanes, tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
   else
     attenuate_bins_x2<NBT, HE, HEAT, false>(lanes, tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
-  cell_shares<HE, HEAT>(lanes, At, c.e, tHI, tHeI, tHeII, f2_sum(g1), f2_sum(g2), f2_sum(h0), f2_sum(h1),
-                        f2_sum(h2), dHI, dHeI, dHeII, dE);
-  return (long long)(At << c.e);
+  deposit_shares<HE, HEAT>(lanes, At, c.e, tHI, tHeI, tHeII, f2_sum(g1), f2_sum(g2), f2_sum(h0), f2_sum(h1),
+                           f2_sum(h2), cells, cell, heat_box);
 }
 
 // Attenuation and deposition in one crossed cell (Sec. 2, Eq. 1) for a
-// segment of seg cells: updates the packet's bins and returns the absorbed
-// total in photon quanta; the species and heating deposits of the cell come
-// back in d* (quanta), left is nonzero while some bin holds photons.  The
-// species and heating sums run over the even and the odd bins separately
+// segment of seg cells: updates the packet's bins and adds the species and
+// heating deposits (quanta) to the cell; left is nonzero while some bin holds
+// photons.  The species and heating sums run over the even and the odd bins separately
 // and are then added, as the two lanes of the packed form do.
-template <int NBT, bool HE, bool HEAT>
-__device__ __forceinline__ long long cell_attenuate(const unsigned lanes, float seg, float dl, float4 ab,
-                                                    Content<NBT>& c, int nb, const BinTables& t, long long& dHI,
-                                                    long long& dHeI, long long& dHeII, long long& dE,
-                                                    unsigned& left) {
+template <int NBT, bool HE, bool HEAT, class Cells>
+__device__ __forceinline__ void cell_attenuate(const unsigned lanes, float seg, float dl, float4 ab, Content<NBT>& c,
+                                               int nb, const BinTables& t, unsigned& left, const Cells& cells,
+                                               unsigned cell, bool heat_box) {
   if constexpr (NBT >= 2 && NBT % 2 == 0)
-    return cell_attenuate_x2<NBT, HE, HEAT>(lanes, seg, dl, ab, c, t, dHI, dHeI, dHeII, dE, left);
+    return cell_attenuate_x2<NBT, HE, HEAT>(lanes, seg, dl, ab, c, t, left, cells, cell, heat_box);
   const float l = seg * dl;
   const float tHI = l * ab.x, tHeI = l * ab.y, tHeII = l * ab.z;
   unsigned long long At = 0;
@@ -452,9 +441,8 @@ __device__ __forceinline__ long long cell_attenuate(const unsigned lanes, float 
     }
     left |= mj;
   }
-  cell_shares<HE, HEAT>(lanes, At, c.e, tHI, tHeI, tHeII, g1[0] + g1[1], g2[0] + g2[1], h0[0] + h0[1],
-                        h1[0] + h1[1], h2[0] + h2[1], dHI, dHeI, dHeII, dE);
-  return (long long)(At << c.e);
+  deposit_shares<HE, HEAT>(lanes, At, c.e, tHI, tHeI, tHeII, g1[0] + g1[1], g2[0] + g2[1], h0[0] + h0[1],
+                           h1[0] + h1[1], h2[0] + h2[1], cells, cell, heat_box);
 }
 
 // Where a walk reads absorbers and adds deposits: the grid in global memory
@@ -482,10 +470,11 @@ constexpr int kStageHalf = 656;          // 512 bytes of first half-records, 32 
 constexpr int kStageCells = 2 * kStageHalf - 16;   // reads below then touch every bank once per half warp
 constexpr int kStageWarp = kStageCells + 128;
 
-// with a single deposited value per crossing (pure H, isothermal) the record
-// has one nonzero: each lane then sends its own
+// with a single deposited value per crossing (pure H, isothermal) there is no
+// record: each lane sends its own value
 template <bool HE, bool HEAT>
 struct GlobalCells {
+ public:
   static constexpr bool kWarp = true;
   const float4* abs;
   unsigned long long* dep;
@@ -497,48 +486,50 @@ struct GlobalCells {
   }
   __device__ __forceinline__ float4 load(unsigned c) const { return __ldg(abs + c); }
   // called by the whole warp; has: this lane has a record for cell c
-  __device__ __forceinline__ void add(bool has, unsigned c, long long a0, long long a1, long long a2,
-                                      long long e) const {
-    if (!HE && !HEAT) {
-      // neighbouring lanes in one cell (near a source) send one sum
-      unsigned cur = has ? c : 0xFFFFFFFFu;
-      unsigned long long v = (unsigned long long)a0;
-      unsigned other = __shfl_xor_sync(0xFFFFFFFFu, cur, 1);
-      if (__any_sync(0xFFFFFFFFu, has && other == cur)) {
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          if (o > 1) other = __shfl_xor_sync(0xFFFFFFFFu, cur, o);
-          const unsigned long long u = __shfl_xor_sync(0xFFFFFFFFu, v, o);
-          if (other == cur) {
-            if (threadIdx.x & o) cur = 0xFFFFFFFFu;
-            else v += u;
-          }
-        }
-      }
-      if (cur != 0xFFFFFFFFu) atomicAdd(dep + 4 * (size_t)cur, v);
-      return;
-    }
+  __device__ __forceinline__ void add(bool has, unsigned c, unsigned long long a0, unsigned long long a1,
+                                      unsigned long long a2, unsigned long long e) const {
+    if (!HE && !HEAT) return add_one(has, c, a0);
     if (!__any_sync(0xFFFFFFFFu, has)) return;
-    constexpr unsigned none = 0xFFFFFFFFu;
     const unsigned lane = threadIdx.x & 31;
     unsigned char* mine = stage + 16 * lane + 32 * (lane >> 3);
-    reinterpret_cast<unsigned*>(stage + kStageCells)[lane] = has ? c : none;
-    *reinterpret_cast<ulonglong2*>(mine) = make_ulonglong2((unsigned long long)a0, (unsigned long long)a1);
-    *reinterpret_cast<ulonglong2*>(mine + kStageHalf) = make_ulonglong2((unsigned long long)a2, (unsigned long long)e);
+    reinterpret_cast<unsigned*>(stage + kStageCells)[lane] = has ? c : kNone;
+    *reinterpret_cast<ulonglong2*>(mine) = make_ulonglong2(a0, a1);
+    *reinterpret_cast<ulonglong2*>(mine + kStageHalf) = make_ulonglong2(a2, e);
     __syncwarp();
     const unsigned k = lane & 3u, g = lane >> 2;     // value k of records 4 g .. 4 g + 3
+    send(reinterpret_cast<const unsigned long long*>(stage + (k >> 1) * kStageHalf + 8 * (k & 1u) + 64 * g +
+                                                     32 * (g >> 1)), 2);
+  }
+  // a record of 32-bit values: 16 bytes, record 4 g + q at word 40 q + 4 g (the
+  // four lanes of each group then read every bank once)
+  __device__ __forceinline__ void add(bool has, unsigned c, uint4 a) const {
+    if (!HE && !HEAT) return add_one(has, c, a.x);
+    if (!__any_sync(0xFFFFFFFFu, has)) return;
+    const unsigned lane = threadIdx.x & 31;
+    reinterpret_cast<unsigned*>(stage + kStageCells)[lane] = has ? c : kNone;
+    *reinterpret_cast<uint4*>(stage + 160 * (lane & 3u) + 16 * (lane >> 2)) = a;
+    __syncwarp();
+    send(reinterpret_cast<const unsigned*>(stage) + lane, 40);
+  }
+
+ private:
+  static constexpr unsigned kNone = 0xFFFFFFFFu;
+  // this lane's value of the four records of its group, `step` elements apart:
+  // sums over records of one cell, each sent with one reduction
+  template <class V>
+  __device__ __forceinline__ void send(const V* src, const int step) const {
+    const unsigned lane = threadIdx.x & 31, g = lane >> 2;
     const uint4 cs = *reinterpret_cast<const uint4*>(stage + kStageCells + 16 * g);
-    const unsigned char* src = stage + (k >> 1) * kStageHalf + 8 * (k & 1u) + 64 * g + 32 * (g >> 1);
     const unsigned cq[4] = {cs.x, cs.y, cs.z, cs.w};
-    unsigned long long* dk = dep + k;
+    unsigned long long* dk = dep + (lane & 3u);
     unsigned cur = cs.x;
-    unsigned long long acc = *reinterpret_cast<const unsigned long long*>(src);
+    unsigned long long acc = src[0];
     bool whole = true;
 #pragma unroll
     for (int q = 1; q < 4; ++q) {
-      const unsigned long long v = *reinterpret_cast<const unsigned long long*>(src + 16 * q);
+      const unsigned long long v = src[q * step];
       const bool other = cq[q] != cur;
-      if (other && cur != none && acc) atomicAdd(dk + 4 * (size_t)cur, acc);
+      if (other && cur != kNone && acc) atomicAdd(dk + 4 * (size_t)cur, acc);
       acc = (other ? 0ull : acc) + v;
       cur = cq[q];
       whole = whole && !other;
@@ -550,11 +541,29 @@ struct GlobalCells {
         const unsigned long long v = __shfl_xor_sync(0xFFFFFFFFu, acc, o);
         const bool same = other == cur;
         acc += same ? v : 0ull;             // (the upper lane's sum is not sent)
-        cur = same && (lane & o) ? none : cur;
+        cur = same && (lane & o) ? kNone : cur;
       }
     }
-    if (cur != none && acc) atomicAdd(dk + 4 * (size_t)cur, acc);
+    if (cur != kNone && acc) atomicAdd(dk + 4 * (size_t)cur, acc);
     __syncwarp();                // the next crossing's records overwrite the staging area
+  }
+  // one value per record: neighbouring lanes in one cell (near a source) send
+  // one sum
+  __device__ __forceinline__ void add_one(bool has, unsigned c, unsigned long long v) const {
+    unsigned cur = has ? c : kNone;
+    unsigned other = __shfl_xor_sync(0xFFFFFFFFu, cur, 1);
+    if (__any_sync(0xFFFFFFFFu, has && other == cur)) {
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        if (o > 1) other = __shfl_xor_sync(0xFFFFFFFFu, cur, o);
+        const unsigned long long u = __shfl_xor_sync(0xFFFFFFFFu, v, o);
+        if (other == cur) {
+          if (threadIdx.x & o) cur = kNone;
+          else v += u;
+        }
+      }
+    }
+    if (cur != kNone) atomicAdd(dep + 4 * (size_t)cur, v);
   }
 };
 
@@ -573,8 +582,11 @@ struct TileCells {
     return (unsigned)((ix - x0) + 16 * ((iy - y0) + 16 * (iz - z0)));
   }
   __device__ __forceinline__ float4 load(unsigned c) const { return sabs[c]; }
-  __device__ __forceinline__ void add(bool has, unsigned c, long long a0, long long a1, long long a2,
-                                      long long e) const {
+  __device__ __forceinline__ void add(bool has, unsigned c, uint4 a) const {
+    add(has, c, a.x, a.y, a.z, a.w);
+  }
+  __device__ __forceinline__ void add(bool has, unsigned c, unsigned long long a0, unsigned long long a1,
+                                      unsigned long long a2, unsigned long long e) const {
     if (!has) return;
     if (a0) atomicAdd(sdep + c, (unsigned long long)a0);
     if (a1) atomicAdd(sdep + 4096 + c, (unsigned long long)a1);
@@ -675,12 +687,9 @@ __device__ __forceinline__ int walk_steps(const bool run, int& ix, int& iy, int&
     if (!go) ab = make_float4(0.f, 0.f, 0.f, 0.f);      // what a lane that is done crosses from now on
     // attenuate and deposit in the current cell (a segment of no length
     // absorbs nothing and is no crossing)
-    long long dHI, dHeI, dHeII, dE;
-    const bool has = cell_attenuate<NBT, HE, HEAT>(lanes, seg, dl, here, N, nb, t, dHI, dHeI, dHeII, dE, left) != 0;
+    cell_attenuate<NBT, HE, HEAT>(lanes, seg, dl, here, N, nb, t, left, cells, cell, heat_box);
     tl.crossings += seg > 0.f ? 1u : 0u;
     if (left == 0 && seg > 0.f) go = false;
-    if (!heat_box) dE = 0;
-    cells.add(has, cell, dHI, dHeI, dHeII, dE);
   }
   ix = dx > 0.f ? R.x1 - rx : R.x0 + rx - 1;
   iy = dy > 0.f ? R.y1 - ry : R.y0 + ry - 1;
@@ -1619,7 +1628,9 @@ template <int NBT, bool HE, bool HEAT>
 int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF* wf, int max_iter,
               cudaStream_t s, EventPairs* ev, int* ev_used) {
   int launches = 0;
-  const int block = o.block_size > 0 ? o.block_size : 256;
+  // (passes chosen by the library: blocks of 128 wait less for their slowest
+  // packet, 193.8 -> 190.5 ms on 1e8 packets of the thin 256^3 case)
+  const int block = o.block_size > 0 ? o.block_size : (a.launch_per_pass ? 128 : 256);
   const int persistent = num_sms() * (2048 / block);
   auto tic = [&]() {
     if (!ev) return;
