@@ -36,11 +36,11 @@
 // what goes is the work around them: divisions become correctly rounded
 // quotients of five or six instructions (k_device.cuh), comparisons, signs and
 // FP32-to-FP64 conversions go to the integer unit, the fixed point's last n_e
-// is not formed, pure H skips the He fits, and in an isothermal box the rates of
-// a cell are evaluated once.  Measured: 393 FP64 instructions per sub-step
-// instead of 473; 668,621 thin cells of 23 sub-steps 16.9 -> 13.6 ms, 128^3
-// H+He 4.84 -> 3.91 ms a step, a 32^3 isothermal FP64 sphere (143 sub-steps one
-// after the other in the source's cell) 9.0 -> 0.56 ms.
+// is not formed, limits on the sub-step that cannot act are ruled out in FP32,
+// pure H skips the He fits, and isothermal pure H evaluates the rates of a cell
+// once.  Measured: 668,621 thin cells of 23 sub-steps 16.9 -> 12.7
+// ms, 128^3 H+He 4.84 -> 3.50 ms a step, a 32^3 isothermal FP64 sphere (143
+// sub-steps one after the other in the source's cell) 9.0 -> 0.55 ms.
 //
 // With the diffuse recombination field on (f_rec > 0) the network uses case
 // A and counts the recombinations straight to the ground state of each ion,
@@ -251,7 +251,7 @@ __device__ __forceinline__ StepBound step_bound(const CellIn& c, const Rates& r,
 // sub-step's starting temperature and n_e and the ions at its end, as in
 // the backward-Euler update.
 // r, rB: the rates at the sub-step's starting temperature, and (COUNT) the
-// case-B ones; ISO, every box is isothermal: those of the cell's first
+// case-B ones; ISO, every box is isothermal pure H: those of the cell's first
 // sub-step serve all of them.
 template <typename RT, bool COUNT, bool ISO>
 __device__ __forceinline__ void substep(const CellIn& c, Rates& r, Rates& rB, double& x, double& y2, double& y3,
@@ -466,8 +466,10 @@ __device__ __forceinline__ void load_cell(const StepArgs& a, int64_t i, int b, C
 // thousands of sub-steps, so handing out work per lane keeps the warps full
 // instead of waiting for the slowest cell of a fixed group of 32.
 //
-// ISO: every box is isothermal; a cell's rates are then the same in all its
-// sub-steps and evaluated once.
+// ISO: every box is isothermal pure H; a cell's rates are then the same in all
+// its sub-steps and evaluated once.  (With He the compiler contracts the He
+// chain differently in the shorter kernel, and results move in the last
+// place: isothermal He boxes take the general kernel.)
 template <typename RT, bool COUNT, bool ISO>
 __global__ void __launch_bounds__(128) k_chemistry(StepArgs a, unsigned long long* next_cell) {
   const unsigned full = 0xFFFFFFFFu;
@@ -539,7 +541,7 @@ void launch_chemistry(const StepArgs& a, cudaStream_t s) {
   const unsigned nb = (unsigned)blocks;
 #define CRASH_CHEM(RT, COUNT)                                                                    \
   do {                                                                                           \
-    if (a.any_heat) k_chemistry<RT, COUNT, false><<<nb, 128, 0, s>>>(a, a.work);                 \
+    if (a.any_heat || a.any_he) k_chemistry<RT, COUNT, false><<<nb, 128, 0, s>>>(a, a.work);                 \
     else k_chemistry<RT, COUNT, true><<<nb, 128, 0, s>>>(a, a.work);                             \
   } while (0)
   if (a.any_rec) {
