@@ -834,6 +834,7 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
     form = transport_form(c, total);
     per_launch = form == FORM_PASSES && !passes_asked(c->opts);
     const int64_t chunk = c->opts.chunk_packets > 0 ? (int64_t)c->opts.chunk_packets : (int64_t)1 << 28;
+    const WFSize have = wavefront_size(c->wf);
     WFSize want;
     if (form == FORM_PASSES) {
       want.queue = std::min<int64_t>(total, chunk);
@@ -842,28 +843,33 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
       want.bundle = std::min<int64_t>(total, chunk);
       want.bundle_keys = std::max<int64_t>(c->n_src_total, std::min<int64_t>(kMaxBundleKeys, want.bundle / 2));
     }
-    const WFSize have = wavefront_size(c->wf);
-    if (c->wf && (have.queue < want.queue || have.bundle < want.bundle || have.bundle_keys < want.bundle_keys)) {
+    bool grow = !c->wf || have.queue < want.queue || have.bundle < want.bundle || have.bundle_keys < want.bundle_keys;
+    if (grow) {
       want.queue = std::max(want.queue, have.queue);       // steps of both forms may alternate
       want.n_keys = want.queue > 0 ? c->n_keys : 0;
       want.bundle = std::max(want.bundle, have.bundle);
       want.bundle_keys = std::max(want.bundle_keys, have.bundle_keys);
-      CK(cudaStreamSynchronize(c->stream));
-      wavefront_destroy(c->wf);
-      c->wf = nullptr;
-      if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
-    }
-    if (!c->wf) {
       const size_t cap = memory_cap();
       const size_t need = (size_t)want.queue * (size_t)(2 * (((32 + 4 * c->n_bins) + 15) / 16 * 16)) +
                           12 * (size_t)std::max(want.queue, want.bundle) + 8 * (size_t)want.bundle_keys;
-      const bool fits = !cap || c->bytes + need <= cap;
-      if (!fits && form != FORM_BUNDLE)
-        return set_err(c, CRASH_ERR_OOM, "device memory cap (CRASH_DEVICE_MEMORY_CAP) exceeded by the packet queue");
+      if (cap && c->bytes + need > cap) {
+        if (form != FORM_BUNDLE)
+          return set_err(c, CRASH_ERR_OOM, "device memory cap (CRASH_DEVICE_MEMORY_CAP) exceeded by the packet queue");
+        form = FORM_DIRECT;           // no room to sort: emission order needs none
+        want = WFSize();
+        grow = !c->wf;
+      }
+    }
+    if (grow) {
+      if (c->wf) {
+        CK(cudaStreamSynchronize(c->stream));
+        wavefront_destroy(c->wf);
+        c->wf = nullptr;
+        if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
+      }
       cudaError_t e = cudaSuccess;
-      if (fits) c->wf = wavefront_create(want, c->n_bins, &e);
+      c->wf = wavefront_create(want, c->n_bins, &e);
       if (!c->wf && form == FORM_BUNDLE) {
-        // no room to sort: emission order needs none
         cudaGetLastError();
         form = FORM_DIRECT;
         c->wf = wavefront_create(WFSize(), c->n_bins, &e);
