@@ -346,6 +346,8 @@ def run_crash(args):
         launch_style = "one thread per packet"
     elif g.get_options()["tile"]:
         launch_style = "tile passes"
+    elif not (g.get_options()["seg_per_iter"] or g.get_options()["resort_interval"]):
+        launch_style = "the library's choice: sorted bundles or passes"
     else:
         launch_style = "one persistent launch per step" if g.get_options()["persistent"] \
             else "one launch per pass"

@@ -1,7 +1,7 @@
 // k_mixed.cu -- mixed-precision transport: FP32 traversal, segment lengths
-// and attenuation, exact int64 photon bookkeeping, FP64 only for the
-// direction draw (so that every packet flies along the same direction as in
-// the FP64 form).
+// and attenuation, exact int64 photon bookkeeping.  The direction draw takes
+// the attempt the FP64 form takes, decided in FP32 and integers, so that every
+// packet flies along the same direction.
 //
 // Per crossed cell and bin j (Sec. 2, Eq. 1): tau_j = l sum_s n_s sigma_s,j;
 // the absorbed count A_j = rint(N_j (1 - e^-tau_j)) <= N_j is an integer and
