@@ -779,6 +779,20 @@ static int transport_form(const crash_ctx* c, int64_t total) {
   if (48 * c->n_cells > l2_bytes() && per_source < 1.25 * n2 && total > c->n_cells / 4) return FORM_PASSES;
   return FORM_BUNDLE;
 }
+// Crossings per packet of the passes the library chooses.  Between two sorts
+// the packets in flight spread, and the more cells a box has the farther the
+// absorbers and deposits they touch outgrow L2; short passes cost more queue
+// traffic and launches.  Thin fields, ms of a step's transport with passes of
+// 64 crossings in blocks of 128 with 64 registers / 48 in blocks of 256 with
+// 80 / 32 with 80: 1e8 packets, 256^3 177 / 191 / 198, 288^3 217 / 229 / 238,
+// 320^3 257 / 260 / 273, 384^3 383 / 319 / 333, 448^3 570 / 436 / 423, 512^3
+// 729 / 578 / 535; 2.5e8 packets, 512^3 1644 / 1258 / 1152.
+static int pass_crossings(const crash_ctx* c) {
+  int64_t most = 0;
+  for (const BoxMeta& m : c->meta) most = std::max(most, m.ncell);
+  return most <= (int64_t)1 << 25 ? kLongPass : most <= (int64_t)1 << 26 ? 48 : 32;
+}
+
 extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t* P) {
   if (!c) return CRASH_ERR_ARG;
   if (!(dt > 0) || !isfinite(dt)) return set_err(c, CRASH_ERR_ARG, "dt must be positive");
@@ -825,14 +839,14 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
   CK(cudaMemcpyAsync(c->d_meta, c->meta.data(), sizeof(BoxMeta) * c->n_boxes,
                      cudaMemcpyHostToDevice, c->stream));
   int form = FORM_DIRECT;
-  bool per_launch = false;
+  int per_launch = 0;
   {
     // workspace: the packet queue (two record buffers) or the sort buffers
     // of the step's form, sized to the step (at most 2^28 packets per chunk:
     // 38 GB of queue with 8 bins, 3.2 GB of sort buffers); none when every
     // packet is traced to the end in emission order.
     form = transport_form(c, total);
-    per_launch = form == FORM_PASSES && !passes_asked(c->opts);
+    per_launch = form == FORM_PASSES && !passes_asked(c->opts) ? pass_crossings(c) : 0;
     const int64_t chunk = c->opts.chunk_packets > 0 ? (int64_t)c->opts.chunk_packets : (int64_t)1 << 28;
     const WFSize have = wavefront_size(c->wf);
     WFSize want;

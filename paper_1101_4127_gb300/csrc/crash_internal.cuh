@@ -83,12 +83,14 @@ struct BinTables {
 //   FORM_PASSES  the packet queue: passes of a few cells with spatial re-sorts,
 //                or tile passes
 enum { FORM_DIRECT = 0, FORM_BUNDLE = 1, FORM_PASSES = 2 };
+// crossings of the longest passes the library chooses (pass_crossings)
+constexpr int kLongPass = 64;
 
 struct StepArgs {
   const BoxMeta* boxes;
   const BoxMeta* boxes_host;      // the same table in host memory (launch code only)
   int form;                       // mixed form: FORM_*
-  int launch_per_pass;            // passes chosen by the library: one launch each, 64 registers
+  int launch_per_pass;            // passes chosen by the library, one launch each: their crossings (0: as asked)
   int n_boxes;
   unsigned long long* step_dev;   // step index (Philox counter word), advanced on the device
   double dt;

@@ -1630,7 +1630,8 @@ int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF
   int launches = 0;
   // (passes chosen by the library: blocks of 128 wait less for their slowest
   // packet, 193.8 -> 190.5 ms on 1e8 packets of the thin 256^3 case)
-  const int block = o.block_size > 0 ? o.block_size : (a.launch_per_pass ? 128 : 256);
+  const bool long_passes = a.launch_per_pass == kLongPass;
+  const int block = o.block_size > 0 ? o.block_size : (long_passes ? 128 : 256);
   const int persistent = num_sms() * (2048 / block);
   auto tic = [&]() {
     if (!ev) return;
@@ -1730,7 +1731,7 @@ int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF
     }
     return launches;
   }
-  const int S = o.seg_per_iter > 0 ? o.seg_per_iter : 64;
+  const int S = o.seg_per_iter > 0 ? o.seg_per_iter : (a.launch_per_pass ? a.launch_per_pass : kLongPass);
   const int R = o.resort_interval == 0 ? 1 : o.resort_interval;
   // emission only writes the packets (no walk): every crossing is made by the
   // passes, which read the queue in sorted order
@@ -1761,7 +1762,7 @@ int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF
     return e == cudaSuccess ? 1 : -1;
   }
   const int nscan = (int)((wf->n_keys + 4095) / 4096);
-  const bool cap64 = o.reg_cap || a.launch_per_pass;
+  const bool cap64 = o.reg_cap || long_passes;
   // the pass p (p >= 1) reads in sorted order when R > 0 and p % R == 0
   auto sorted_pass = [&](int p) { return p >= 1 && p < passes && R > 0 && (p % R) == 0; };
   for (int64_t g0 = 0; g0 < a.total_packets; g0 += wf->cap) {

@@ -108,6 +108,35 @@ def test_large_grid_passes_equal_emission_order():
     h.close()
 
 
+@pytest.mark.parametrize("dims,n_src,per_src,crossings", [
+    ((512, 256, 256), 100, 85000, 64),               # 2^25 cells
+    ((512, 256, 257), 100, 85000, 48),
+    ((512, 512, 257), 150, 113000, 32),
+])
+def test_pass_length_by_grid_size(dims, n_src, per_src, crossings):
+    """Larger boxes take shorter passes by default; the bits are those of
+    emission order."""
+    rng = np.random.default_rng(6)
+    E, f = inputs.blackbody_bins(1e5)
+    box = inputs.Box(n=512, box_cm=6.6 * inputs.KPC_CM * 4, nH=None, nH0=1e-3, he_over_h=0.08, x_HII0=1.2e-3,
+                     x_HeII0=0.0, x_HeIII0=0.0, T0=1e4, isothermal=0, caseB=1, z_compton=9.0, seed=743,
+                     src_pos=rng.uniform(0, 1, (n_src, 3)) * np.array(dims), src_ndot=rng.uniform(1e47, 1e49, n_src),
+                     bin_eV=E, bin_frac=np.tile(f, (n_src, 1)), dims=dims)
+    out = []
+    for opts in ({}, dict(wavefront=0)):
+        g = native.Grid(box, native.CRASH_MIXED)
+        g.set_options(chemistry=0, **opts)
+        before = g.launch_count()
+        g.step(DT, n_src * per_src)
+        launches = g.launch_count() - before
+        out.append([g.read(f_) for f_ in (native.F_DEP_HI, native.F_DEP_E, native.F_BUDGET)])
+        g.close()
+        if not opts:       # every pass but the last sorts (four launches); the walk crosses at most the three edges
+            passes = -(-(sum(dims) + 3) // crossings) + 1
+            assert 5 * passes - 4 <= launches <= 5 * passes + 8
+    _same(*out, "passes")
+
+
 @pytest.mark.parametrize("per_src", [7, 30000, 260000])
 def test_noalloc_bundles_equal_emission_order(per_src):
     """The allocation-free call: all at once, one bundle chunk, several."""
