@@ -857,7 +857,9 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
       want.bundle = std::min<int64_t>(total, chunk);
       want.bundle_keys = std::max<int64_t>(c->n_src_total, std::min<int64_t>(kMaxBundleKeys, want.bundle / 2));
     }
-    bool grow = !c->wf || have.queue < want.queue || have.bundle < want.bundle || have.bundle_keys < want.bundle_keys;
+    // (new sources may change the number of colours, and with it the length of a record)
+    bool grow = !c->wf || have.queue < want.queue || have.bundle < want.bundle || have.bundle_keys < want.bundle_keys ||
+                (want.queue > 0 && have.nb != c->n_bins);
     if (grow) {
       want.queue = std::max(want.queue, have.queue);       // steps of both forms may alternate
       want.n_keys = want.queue > 0 ? c->n_keys : 0;

@@ -176,9 +176,11 @@ int launch_trace_mixed_external(StepArgs a, const BinTables& t, const crash_run_
 void cross_sections(int nb, const double* E, BinTables& t, int& heatF);
 
 // Mixed-form workspace: packets of the queue, packets of a bundle chunk, sort
-// keys of the queue's passes and direction keys of the bundles.
+// keys of the queue's passes and direction keys of the bundles; nb, the
+// colours of the queue's records (their length follows from it).
 struct WFSize {
   int64_t queue = 0, bundle = 0, n_keys = 0, bundle_keys = 0;
+  int nb = 0;
 };
 void* wavefront_create(const WFSize& n, int n_bins, cudaError_t* err);
 void wavefront_destroy(void* w);

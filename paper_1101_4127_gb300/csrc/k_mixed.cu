@@ -1918,7 +1918,7 @@ WFSize wavefront_size(void* p) {
   WFSize n;
   if (p) {
     const WF* w = (const WF*)p;
-    n = {w->cap, w->bcap, w->n_keys, w->bkeys};
+    n = {w->cap, w->bcap, w->n_keys, w->bkeys, w->nb};
   }
   return n;
 }
