@@ -228,6 +228,7 @@ __device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
 }
 
 enum { ALIVE = 0, ABSORBED = 1, ESCAPED = 2 };
+constexpr unsigned kFull = 0xFFFFFFFFu;      // every lane of a warp
 
 // One bin of optical depth tau >= 0.5: the transmitted part is rounded and
 // the absorbed count is the rest, as in absorb(); q is replaced.
@@ -262,9 +263,9 @@ __device__ __forceinline__ unsigned absorb_thick(unsigned m, float Nf, float tau
 // so that lanes in thin and in thick cells share one instruction stream; and a
 // pair that holds no photons in any lane (soft bins die within the first thick
 // cells) is left out: it absorbs nothing and adds nothing.
-// lanes: the lanes that call together.
+// (Called by whole warps.)
 template <int NBT, bool HE, bool HEAT, bool THIN>
-__device__ __forceinline__ void attenuate_bins_x2(const unsigned lanes, const f32x2 tHI2, const f32x2 tHeI2, const f32x2 tHeII2,
+__device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 tHeI2, const f32x2 tHeII2,
                                                   Content<NBT>& c, const BinTables& t,
                                                   unsigned long long& At, unsigned& left, f32x2& g1,
                                                   f32x2& g2, f32x2& h0, f32x2& h1, f32x2& h2) {
@@ -272,7 +273,7 @@ __device__ __forceinline__ void attenuate_bins_x2(const unsigned lanes, const f3
 #pragma unroll
   for (int j = 0; j < NBT; j += 2) {
     const unsigned m0 = c.m[j], m1 = c.m[j + 1];
-    if (!THIN && !__any_sync(lanes, (m0 | m1) != 0u)) continue;
+    if (!THIN && !__any_sync(kFull, (m0 | m1) != 0u)) continue;
     const float4 t01 = t.pairs[0][j / 2], t23 = t.pairs[1][j / 2], t45 = t.pairs[2][j / 2];
     const f32x2 s0 = f2(t01.x, t01.y);
     f32x2 tau = f2_mul(tHI2, s0);
@@ -301,7 +302,7 @@ __device__ __forceinline__ void attenuate_bins_x2(const unsigned lanes, const f3
       f2_split(tau, tau0, tau1);
       // (not below 0.5: NaN, an infinite opacity times 0, absorbs everything)
       const bool thick0 = !(tau0 < 0.5f), thick1 = !(tau1 < 0.5f);
-      if (__any_sync(lanes, thick0 || thick1)) {
+      if (__any_sync(kFull, thick0 || thick1)) {
         float q0, q1, p0, p1;
         f2_split(q2, q0, q1);
         const unsigned B0 = absorb_thick(m0, N0, tau0, p0), B1 = absorb_thick(m1, N1, tau1, p1);
@@ -342,7 +343,7 @@ __device__ __forceinline__ float f2_sum(f32x2 v) {
 // while no lane absorbs 2^31 quanta the shares are 32-bit numbers, one
 // conversion each is the whole rounding, and the record is half as long.
 template <bool HE, bool HEAT, class Cells>
-__device__ __forceinline__ void deposit_shares(const unsigned lanes, unsigned long long At, int e, float tHI, float tHeI,
+__device__ __forceinline__ void deposit_shares(unsigned long long At, int e, float tHI, float tHeI,
                                                float tHeII, float G1, float G2, float H0, float H1, float H2,
                                                const Cells& cells, unsigned cell, bool heat_box) {
   const unsigned long long Au = At << e;
@@ -351,13 +352,13 @@ __device__ __forceinline__ void deposit_shares(const unsigned lanes, unsigned lo
   const float fHeI = HE ? tHeI * G1 : 0.f, fHeII = HE ? tHeII * G2 : 0.f;
   const float fheat = HEAT ? (HE ? fmaf(tHeII, H2, fmaf(tHeI, H1, tHI * H0)) : tHI * H0) : 0.f;
   const float x1 = fHeI * unit, x2 = fHeII * unit, xh = heat_box ? fheat * unit : 0.f;
-  if (!__any_sync(lanes, Au >= 0x80000000ull)) {
+  if (!__any_sync(kFull, Au >= 0x80000000ull)) {
     const unsigned A = (unsigned)Au;
     unsigned a1 = HE ? __float2uint_rn(x1) : 0u, a2 = HE ? __float2uint_rn(x2) : 0u;
     const unsigned h = HEAT ? __float2uint_rn(xh) : 0u;
     // He shares above the cell's total only by rounding: clamp then (the
     // clamps change nothing when the two fit; neither nears 2^32)
-    if (HE && __any_sync(lanes, (unsigned long long)a1 + a2 > A)) {
+    if (HE && __any_sync(kFull, (unsigned long long)a1 + a2 > A)) {
       a1 = a1 > A ? A : a1;
       a2 = a2 > A - a1 ? A - a1 : a2;
     }
@@ -365,7 +366,7 @@ __device__ __forceinline__ void deposit_shares(const unsigned lanes, unsigned lo
   } else {
     unsigned long long a1 = HE ? float_to_ull(x1) : 0ull, a2 = HE ? float_to_ull(x2) : 0ull;
     const unsigned long long h = HEAT ? float_to_ull(xh) : 0ull;
-    if (HE && __any_sync(lanes, a1 + a2 > Au)) {
+    if (HE && __any_sync(kFull, a1 + a2 > Au)) {
       a1 = a1 > Au ? Au : a1;
       a2 = a2 > Au - a1 ? Au - a1 : a2;
     }
@@ -376,7 +377,7 @@ __device__ __forceinline__ void deposit_shares(const unsigned lanes, unsigned lo
 // left: on entry, nonzero if some bin holds photons; on return, the same
 // after the cell
 template <int NBT, bool HE, bool HEAT, class Cells>
-__device__ __forceinline__ void cell_attenuate_x2(const unsigned lanes, float seg, float dl, float4 ab, Content<NBT>& c,
+__device__ __forceinline__ void cell_attenuate_x2(float seg, float dl, float4 ab, Content<NBT>& c,
                                                   const BinTables& t, unsigned& left, const Cells& cells,
                                                   unsigned cell, bool heat_box) {
   static_assert(NBT >= 2 && NBT % 2 == 0, "bin pairs");
@@ -390,11 +391,11 @@ __device__ __forceinline__ void cell_attenuate_x2(const unsigned lanes, float se
   const float k0max = tHI * t.sigma32_max[0];
   const float tau_max = HE ? fmaf(tHeII, t.sigma32_max[2], fmaf(tHeI, t.sigma32_max[1], k0max)) : k0max;
   // (either form gives a lane in a thin cell the same bits: the vote only picks the instruction stream)
-  if (!__any_sync(lanes, !(tau_max < 0.5f)))
-    attenuate_bins_x2<NBT, HE, HEAT, true>(lanes, tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
+  if (!__any_sync(kFull, !(tau_max < 0.5f)))
+    attenuate_bins_x2<NBT, HE, HEAT, true>(tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
   else
-    attenuate_bins_x2<NBT, HE, HEAT, false>(lanes, tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
-  deposit_shares<HE, HEAT>(lanes, At, c.e, tHI, tHeI, tHeII, f2_sum(g1), f2_sum(g2), f2_sum(h0), f2_sum(h1),
+    attenuate_bins_x2<NBT, HE, HEAT, false>(tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
+  deposit_shares<HE, HEAT>(At, c.e, tHI, tHeI, tHeII, f2_sum(g1), f2_sum(g2), f2_sum(h0), f2_sum(h1),
                            f2_sum(h2), cells, cell, heat_box);
 }
 
@@ -404,11 +405,11 @@ __device__ __forceinline__ void cell_attenuate_x2(const unsigned lanes, float se
 // photons.  The species and heating sums run over the even and the odd bins separately
 // and are then added, as the two lanes of the packed form do.
 template <int NBT, bool HE, bool HEAT, class Cells>
-__device__ __forceinline__ void cell_attenuate(const unsigned lanes, float seg, float dl, float4 ab, Content<NBT>& c,
+__device__ __forceinline__ void cell_attenuate(float seg, float dl, float4 ab, Content<NBT>& c,
                                                int nb, const BinTables& t, unsigned& left, const Cells& cells,
                                                unsigned cell, bool heat_box) {
   if constexpr (NBT >= 2 && NBT % 2 == 0)
-    return cell_attenuate_x2<NBT, HE, HEAT>(lanes, seg, dl, ab, c, t, left, cells, cell, heat_box);
+    return cell_attenuate_x2<NBT, HE, HEAT>(seg, dl, ab, c, t, left, cells, cell, heat_box);
   const float l = seg * dl;
   const float tHI = l * ab.x, tHeI = l * ab.y, tHeII = l * ab.z;
   unsigned long long At = 0;
@@ -441,7 +442,7 @@ __device__ __forceinline__ void cell_attenuate(const unsigned lanes, float seg, 
     }
     left |= mj;
   }
-  deposit_shares<HE, HEAT>(lanes, At, c.e, tHI, tHeI, tHeII, g1[0] + g1[1], g2[0] + g2[1], h0[0] + h0[1],
+  deposit_shares<HE, HEAT>(At, c.e, tHI, tHeI, tHeII, g1[0] + g1[1], g2[0] + g2[1], h0[0] + h0[1],
                            h1[0] + h1[1], h2[0] + h2[1], cells, cell, heat_box);
 }
 
@@ -475,7 +476,7 @@ constexpr int kStageWarp = kStageCells + 128;
 template <bool HE, bool HEAT>
 struct GlobalCells {
  public:
-  static constexpr bool kWarp = true;
+  static constexpr bool kHold = false;
   const float4* abs;
   unsigned long long* dep;
   unsigned coff, ny, nz;         // ny, nz: cells from a row, and from a plane, to the next
@@ -573,7 +574,7 @@ struct GlobalCells {
 // one array of 4096 per species (so that lanes at different cells spread
 // over the banks), and go to the grid once per work item
 struct TileCells {
-  static constexpr bool kWarp = false;
+  static constexpr bool kHold = true;
   static constexpr unsigned ny = 16, nz = 256;
   const float4* sabs;              // shared, [16][16][16]
   unsigned long long* sdep;        // shared, [4][16][16][16]
@@ -614,9 +615,9 @@ struct Region {
 // rest of c dt) is used up, the last segment cut there (Sec. 2 periodic
 // boxes).  The photons the walk absorbed are counted once at its end, as the
 // drop of the packet's content.
-// run: the lane has a packet.  With Cells::kWarp the whole warp walks
-// together (every lane calls, and lanes whose packet is done wait for the
-// last) because the warp sends its deposits together.
+// run: the lane has a packet.  The whole warp walks together: every lane
+// calls, and lanes whose packet is done wait for the last, because the warp
+// sends its deposits together and its branches are votes of all lanes.
 template <int NBT, bool HE, bool HEAT, bool PER, class Cells>
 __device__ __forceinline__ int walk_steps(const bool run, int& ix, int& iy, int& iz, float& tMx, float& tMy, float& tMz,
                                     const float dx, const float dy, const float dz, Content<NBT>& N,
@@ -649,15 +650,16 @@ __device__ __forceinline__ int walk_steps(const bool run, int& ix, int& iy, int&
   // A lane that is done goes on with segments of no length, which absorb
   // nothing, load nothing and are no crossings: the warp stays in one
   // instruction stream, whose branches are votes of all lanes.  (Its step
-  // counts move on past the face it left through, or no longer matter.)
+  // counts move on past the face it left through, or no longer matter; with
+  // Cells::kHold, where a packet that leaves goes on elsewhere, it stays.)
   for (int it = 1;; ++it) {
-    if (Cells::kWarp ? !__any_sync(0xFFFFFFFFu, go) : !go) break;
-    const unsigned lanes = Cells::kWarp ? 0xFFFFFFFFu : __activemask();
+    if (!__any_sync(kFull, go)) break;
     const unsigned cell = next;
     // step the walk into the next cell (ties x before y before z) and request
     // its absorbers
-    float seg = fminf(tMx, fminf(tMy, tMz));
-    const bool bx = tMx == seg, by = !bx && tMy == seg, bz = !bx && !by;
+    const bool hold = Cells::kHold && !go;
+    float seg = hold ? 0.f : fminf(tMx, fminf(tMy, tMz));
+    const bool bx = !hold && tMx == seg, by = !hold && !bx && tMy == seg, bz = !hold && !bx && !by;
     tMx = bx ? tDx : tMx - seg;
     tMy = by ? tDy : tMy - seg;
     tMz = bz ? tDz : tMz - seg;
@@ -687,7 +689,7 @@ __device__ __forceinline__ int walk_steps(const bool run, int& ix, int& iy, int&
     if (!go) ab = make_float4(0.f, 0.f, 0.f, 0.f);      // what a lane that is done crosses from now on
     // attenuate and deposit in the current cell (a segment of no length
     // absorbs nothing and is no crossing)
-    cell_attenuate<NBT, HE, HEAT>(lanes, seg, dl, here, N, nb, t, left, cells, cell, heat_box);
+    cell_attenuate<NBT, HE, HEAT>(seg, dl, here, N, nb, t, left, cells, cell, heat_box);
     tl.crossings += seg > 0.f ? 1u : 0u;
     if (left == 0 && seg > 0.f) go = false;
   }
@@ -1366,14 +1368,14 @@ __global__ void __launch_bounds__(kTileBlock, 1) k_tile_pass(StepArgs a, BinTabl
       bool alive = false;
       int ix = 0, iy = 0, iz = 0;
       float tMx = 0.f, tMy = 0.f, tMz = 0.f, fx = 0.f, fy = 0.f, fz = 0.f;
-      Content<NBT> N;
-      N.e = 0;
-      if (j < hi) {
+      Content<NBT> N{};
+      if (j < hi)
         load_record<NBT>(w.rec_in, w.rs, (long long)w.perm[j], ix, iy, iz, pb, tMx, tMy, tMz, fx, fy, fz,
                          N, nb);
-        const Region R{x0, y0, z0, x0 + ex, y0 + ey, z0 + ez};
-        const int r = walk<NBT, HE, HEAT, false>(true, ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, R, cells, t, nb, 64,
-                                                 tl);
+      const Region R{x0, y0, z0, x0 + ex, y0 + ey, z0 + ez};
+      const int r = walk<NBT, HE, HEAT, false>(j < hi, ix, iy, iz, tMx, tMy, tMz, fx, fy, fz, N, M, R, cells, t, nb, 64,
+                                               tl);
+      if (j < hi) {
         if (r == ESCAPED) tl.escaped += N.total(nb);
         alive = (r == ALIVE);
       }
