@@ -260,12 +260,13 @@ __device__ __forceinline__ unsigned absorb_thick(unsigned m, float Nf, float tau
 // bin is looked at on its own, and the packet's liveness is unchanged (left
 // is not recomputed).  Otherwise every bin pair is done by the series first
 // and, if any lane has a thick bin in it, both ways, each lane taking its own,
-// so that lanes in thin and in thick cells share one instruction stream; and a
-// pair that holds no photons in any lane (soft bins die within the first thick
-// cells) is left out: it absorbs nothing and adds nothing.
+// so that lanes in thin and in thick cells share one instruction stream (thick:
+// this lane's cell may hold a thick bin; without it every bin takes the
+// series); and a pair that holds no photons in any lane (soft bins die within
+// the first thick cells) is left out: it absorbs nothing and adds nothing.
 // (Called by whole warps.)
 template <int NBT, bool HE, bool HEAT, bool THIN>
-__device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 tHeI2, const f32x2 tHeII2,
+__device__ __forceinline__ void attenuate_bins_x2(const bool thick, const f32x2 tHI2, const f32x2 tHeI2, const f32x2 tHeII2,
                                                   Content<NBT>& c, const BinTables& t,
                                                   unsigned long long& At, unsigned& left, f32x2& g1,
                                                   f32x2& g2, f32x2& h0, f32x2& h1, f32x2& h2) {
@@ -301,7 +302,7 @@ __device__ __forceinline__ void attenuate_bins_x2(const f32x2 tHI2, const f32x2 
       float tau0, tau1;
       f2_split(tau, tau0, tau1);
       // (not below 0.5: NaN, an infinite opacity times 0, absorbs everything)
-      const bool thick0 = !(tau0 < 0.5f), thick1 = !(tau1 < 0.5f);
+      const bool thick0 = thick && !(tau0 < 0.5f), thick1 = thick && !(tau1 < 0.5f);
       if (__any_sync(kFull, thick0 || thick1)) {
         float q0, q1, p0, p1;
         f2_split(q2, q0, q1);
@@ -390,11 +391,15 @@ __device__ __forceinline__ void cell_attenuate_x2(float seg, float dl, float4 ab
   // largest cross sections in the same operation order (rounding is monotone)
   const float k0max = tHI * t.sigma32_max[0];
   const float tau_max = HE ? fmaf(tHeII, t.sigma32_max[2], fmaf(tHeI, t.sigma32_max[1], k0max)) : k0max;
-  // (either form gives a lane in a thin cell the same bits: the vote only picks the instruction stream)
-  if (!__any_sync(kFull, !(tau_max < 0.5f)))
-    attenuate_bins_x2<NBT, HE, HEAT, true>(tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
+  // A segment of no length (a packet that starts on a face or meets an edge)
+  // absorbs nothing, whatever its cell holds: 0 times an infinite absorber is
+  // NaN, and all its bins take the series, which sends nothing.
+  const bool thick = seg > 0.f && !(tau_max < 0.5f);
+  // (either form gives a lane without thick bins the same bits: the vote only picks the instruction stream)
+  if (!__any_sync(kFull, thick))
+    attenuate_bins_x2<NBT, HE, HEAT, true>(false, tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
   else
-    attenuate_bins_x2<NBT, HE, HEAT, false>(tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
+    attenuate_bins_x2<NBT, HE, HEAT, false>(thick, tHI2, tHeI2, tHeII2, c, t, At, left, g1, g2, h0, h1, h2);
   deposit_shares<HE, HEAT>(At, c.e, tHI, tHeI, tHeII, f2_sum(g1), f2_sum(g2), f2_sum(h0), f2_sum(h1),
                            f2_sum(h2), cells, cell, heat_box);
 }
@@ -421,7 +426,7 @@ __device__ __forceinline__ void cell_attenuate(float seg, float dl, float4 ab, C
     float tau = tHI * t.sigma32[0][j];
     if (HE) tau = fmaf(tHeII, t.sigma32[2][j], fmaf(tHeI, t.sigma32[1][j], tau));
     unsigned mj = c.m[j];
-    if (mj > 0u) {
+    if (mj > 0u && seg > 0.f) {
       float q;
       const unsigned A = absorb(mj, tau, q);
       mj -= A;

@@ -1,0 +1,74 @@
+"""Absorbers and fractions outside the ordinary range.  An infinite absorber is
+a perfect sink of the packets that cross it and of no others: a segment of no
+length (a source on a cell's corner starts one in the cell above it for every
+packet that flies the other way) absorbs nothing."""
+import ctypes as C
+import itertools
+
+import numpy as np
+import pytest
+
+from paper_1101_4127_gb300 import inputs, native
+from _common import small_hhe_box
+
+pytestmark = pytest.mark.gpu
+DEPOSITS = [native.F_DEP_HI, native.F_DEP_HEI, native.F_DEP_HEII, native.F_DEP_E, native.F_BUDGET]
+DT = 0.01 * inputs.MYR_S
+
+
+def _bins(n):
+    return np.array([20.0]) if n == 1 else np.geomspace(14.0, 150.0, n)
+
+
+@pytest.mark.parametrize("bins,packets", list(itertools.product((1, 5, 8), (4000, 200000))))
+def test_segment_of_no_length_in_an_infinite_absorber(bins, packets):
+    """The sink's deposits equal those of an absorber of a finite density that
+    lets nothing through (optical depths above 1e9)."""
+    torch = pytest.importorskip("torch")
+    box = small_hhe_box((8, 8, 8), n_src=1, seed=810)
+    arrays = [np.ascontiguousarray(a, np.float64).reshape(-1) for a in
+              (np.array([4.0, 4.0, 4.0]), box.src_ndot, _bins(bins), np.full(bins, 1.0 / bins))]
+    pos, ndot, E, f = (a.ctypes.data_as(C.POINTER(C.c_double)) for a in arrays)
+    sink = 4 + 8 * (4 + 8 * 4)
+    got = []
+    for density in (np.inf, 1e25):
+        a = torch.full((512, 4), 1e-7, dtype=torch.float32, device="cuda")
+        a[sink, 0] = density
+        a[sink, 1:] = 0.0
+        dep = torch.zeros((512, 4), dtype=torch.int64, device="cuda")
+        torch.cuda.synchronize()
+        budget = np.zeros(8, np.int64)
+        desc = native.make_desc(box, native.CRASH_MIXED)
+        st = native.lib().crash_transport_noalloc(C.byref(desc), 1, pos, ndot, bins, E, f, DT, 0, packets, 0, a.data_ptr(),
+                                                  dep.data_ptr(), budget.ctypes.data_as(C.POINTER(C.c_int64)), None)
+        assert st == native.CRASH_OK
+        dep = dep.cpu().numpy()
+        # (an infinite optical depth has no heating share; the photons and every other cell are the same)
+        dep[sink, 3] = 0
+        got.append((dep, budget[:5].copy()))
+    (d0, b0), (d1, b1) = got
+    assert np.array_equal(b0, b1) and b0[0] == b0[1] + b0[2] and b0[2] > 0.8 * b0[0]
+    assert np.array_equal(d0, d1) and d0[sink, 0] > 0.1 * b0[0]
+
+
+@pytest.mark.parametrize("field,value", [(native.F_XHEII, 4.5), (native.F_XHII, 1.5)])
+def test_negative_absorbers_do_not_depend_on_the_order(field, value):
+    """Fractions above 1 make absorbers negative; the deposits are the same in
+    emission order, in bundles, in passes and in tiles."""
+    box = small_hhe_box((20, 20, 20), n_src=2, seed=811)
+    P = 2 * 70001
+    rng = np.random.default_rng(1)
+    sel = rng.choice(8000, 300, replace=False)
+    out = []
+    for opts in (dict(wavefront=0), dict(), dict(seg_per_iter=8), dict(tile=1)):
+        g = native.Grid(box, native.CRASH_MIXED)
+        g.set_options(chemistry=0, **opts)
+        x = g.read(field)
+        x.reshape(-1)[sel] = value
+        g.write(field, x)
+        g.step(DT, P)
+        out.append([g.read(k) for k in DEPOSITS])
+        g.close()
+    for o in out[1:]:
+        for a, b in zip(out[0], o):
+            assert np.array_equal(a, b)
