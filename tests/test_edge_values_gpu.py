@@ -72,3 +72,29 @@ def test_negative_absorbers_do_not_depend_on_the_order(field, value):
     for o in out[1:]:
         for a, b in zip(out[0], o):
             assert np.array_equal(a, b)
+
+
+def test_fp64_thick_cells_with_fractions_above_one():
+    """FP64 form: cells with x_HII = 1.5 dense enough that e^-tau overflows are
+    transparent (the transmitted photons are clamped to those that entered):
+    they absorb nothing and the photon budget closes."""
+    box = small_hhe_box((12, 12, 12), n_src=2, seed=812)
+    sel = np.random.default_rng(2).choice(1728, 80, replace=False)
+    box.nH = box.nH.copy()
+    box.nH.reshape(-1)[sel] = 1e6
+    g = native.Grid(box, native.CRASH_FP64_PLAIN)
+    g.set_options(chemistry=0)
+    x = g.read(native.F_XHII)
+    x.reshape(-1)[sel] = 1.5
+    g.write(native.F_XHII, x)
+    for f, v in ((native.F_XHEII, 0.0), (native.F_XHEIII, 1.0)):      # no He absorbers there either
+        y = g.read(f)
+        y.reshape(-1)[sel] = v
+        g.write(f, y)
+    g.step(DT, 2 * 6000)
+    b = g.read(native.F_BUDGET)
+    assert b[0] == b[1] + b[2] and 0 < b[1] <= b[0]
+    for f in DEPOSITS[:4]:
+        d = g.read(f).reshape(-1)
+        assert (d >= 0).all() and (d[sel] == 0).all()
+    g.close()
