@@ -208,6 +208,8 @@ __device__ __forceinline__ void walk_fp64(const StepArgs& a, const BinTables& t,
         nHeI = a01.y;
         nHeII = __ldg(reinterpret_cast<const double2*>(a.abs64) + 2 * cell + 1).x;
       }
+      // (He absorbers that are not finite count in every bin: 0 times them is NaN)
+      const bool odd = HE && (not_finite(nHeI) || not_finite(nHeII));
       long long dHI = 0, dHeI = 0, dHeII = 0, left = 0;
       double heat = 0.0;
 #pragma unroll
@@ -219,7 +221,7 @@ __device__ __forceinline__ void walk_fp64(const StepArgs& a, const BinTables& t,
         if (Nj == 0) continue;
         const double kHI = nHI * t.sigma[0][j];
         double kap = kHI, kHeI = 0.0, kHeII = 0.0;
-        const bool he1 = HE && t.sigma[1][j] > 0.0, he2 = HE && t.sigma[2][j] > 0.0;
+        const bool he1 = HE && (t.sigma[1][j] > 0.0 || odd), he2 = HE && (t.sigma[2][j] > 0.0 || odd);
         if (he1) {
           kHeI = nHeI * t.sigma[1][j];
           kap = kap + kHeI;

@@ -98,3 +98,28 @@ def test_fp64_thick_cells_with_fractions_above_one():
         d = g.read(f).reshape(-1)
         assert (d >= 0).all() and (d[sel] == 0).all()
     g.close()
+
+
+def test_fp64_he_absorbers_that_are_not_numbers():
+    """FP64 form: a cell whose He absorbers are NaN takes every photon that
+    enters it, of the colours below the He thresholds too, as a cell of
+    infinite H I does."""
+    box = small_hhe_box((12, 12, 12), n_src=2, seed=813, thin=True)
+    sel = np.random.default_rng(3).choice(1728, 80, replace=False)
+    out = []
+    for field, value in ((native.F_XHEII, np.nan), (native.F_XHII, -np.inf)):
+        g = native.Grid(box, native.CRASH_FP64_PLAIN)
+        g.set_options(chemistry=0)
+        x = g.read(field)
+        x.reshape(-1)[sel] = value
+        g.write(field, x)
+        g.step(DT, 2 * 6000)
+        b = g.read(native.F_BUDGET)
+        assert b[0] == b[1] + b[2] and b[1] > 0 and b[2] > 0
+        dep = [g.read(f).reshape(-1) for f in DEPOSITS[:4]]
+        for d in dep:
+            d[sel] = 0
+        out.append(dep + [b[:5]])
+        g.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
