@@ -766,17 +766,29 @@ static int transport_form(const crash_ctx* c, int64_t total) {
   if (c->n_src_total > kMaxBundleKeys) return c->any_periodic ? FORM_DIRECT : FORM_PASSES;
   if (c->any_periodic) return FORM_BUNDLE;
   // A bundle's 32 packets spread to about w cells at half the grid's width,
-  // w^2 = (n / 2)^2 4 pi 32 / (packets per source).  Where absorbers and
-  // deposits (48 bytes a cell) do not fit L2, wide bundles miss it, and passes
-  // in spatial order win if they have packets enough to fill their buckets:
-  // 20e6 packets, thin, ms for bundles / passes: 192^3 2000 sources (w = 19)
-  // 54 / 40, 1000 sources of 60e6 (8) 118 / 117, 300 (7) 39 / 41, 1 source 35
-  // / 45; 256^3 2000 sources (26) 78 / 52, 100 (6) 45 / 51; 1e6 packets, 1000
-  // sources (81) 5.7 / 6.9.  128^3 fits L2: 2000 sources (13) 25.5 / 25.6.
+  // w^2 = (n / 2)^2 4 pi 32 / (packets per source).  The wider the bundles, the
+  // less their lanes and their neighbours share of absorbers and deposits (48
+  // bytes a cell), and where these do not fit L2 they miss it too; passes in
+  // spatial order cost their sorts and win if there are packets enough to pay
+  // for these and to fill the buckets.  8 colours, thin, ms for bundles / passes
+  // (sources x packets per source, w): 128^3 300 x 67,000 (5) 19.9 / 20.4, 1000
+  // x 60,000 (5) 58.6 / 58.7, 10,000 x 600 (52) 9.5 / 7.0, 10^6 x 6 (524) 14.1 /
+  // 7.2; 160^3 300 x 67,000 (6) 27.6 / 25.4, 1000 x 60,000 (7) 82.6 / 71.7;
+  // 256^3 30 x 200,000 (6) 13.2 / 14.7, 300 x 200,000 (6) 138 / 116, 300 x 8,300
+  // (28) 12.6 / 9.6, 10^5 x 60 (331) 41.1 / 16.9; by number, 10^5 sources: 10^6
+  // packets 256^3 7.8 / 6.7, 320^3 10.7 / 10.4, 512^3 19.7 / 23.7; 512^3 2.5e6
+  // packets 43.4 / 44.1, 6e6 98.3 / 79.3.  Over 698 steps of 1 to 64 boxes, thin
+  // and thick, the rule's form takes 1.24 times the other's time at most and
+  // 1.003 of the faster one's in the mean; none of 1, 3 or 16 colours (225
+  // steps) is slower than before there were bundles.  (A batch counts as one
+  // field: its packets are in flight in many boxes at once.)
   int64_t most = 0;
   for (const BoxMeta& m : c->meta) most = std::max(most, m.ncell);
-  const double n2 = pow((double)most, 2.0 / 3.0), per_source = (double)total / (double)c->n_src_total;
-  if (48 * c->n_cells > l2_bytes() && per_source < 1.25 * n2 && total > c->n_cells / 4) return FORM_PASSES;
+  const double per_source = (double)total / (double)c->n_src_total;
+  const double w = sqrt(32.0 * 3.14159265358979 * pow((double)most, 2.0 / 3.0) / per_source);
+  const double fill = std::min(1.0, (double)total / (double)c->n_cells);
+  const double narrow = (48 * c->n_cells > l2_bytes() ? 5.0 : 16.0) / sqrt(fill);
+  if (w > narrow && total >= std::max<int64_t>(1 << 19, c->n_cells / 48)) return FORM_PASSES;
   return FORM_BUNDLE;
 }
 // Crossings per packet of the passes the library chooses.  Between two sorts
