@@ -174,8 +174,15 @@ typedef struct {
 void crash_default_opts(crash_run_opts* o);
 
 /* Device memory of a context may be capped with the environment variable
-   CRASH_DEVICE_MEMORY_CAP (bytes): creation, sources or a step whose
-   allocations would exceed it fail with CRASH_ERR_OOM and allocate nothing. */
+   CRASH_DEVICE_MEMORY_CAP (bytes; the sources' tables, 440 bytes each, are not
+   counted): a creation whose allocations would exceed it fails with
+   CRASH_ERR_OOM and allocates nothing.  A step (either form) allocates its
+   packet workspace on first use and when it grows: the queue of its passes, or
+   the sort buffers of its bundles (12 bytes a packet and 8 a direction key).
+   Where that has no room, under the cap or on the
+   device, a step whose form the library chooses runs in bundles or in emission
+   order instead, with the same results; passes that were asked for (see
+   wavefront) fail with CRASH_ERR_OOM. */
 
 /* Create a context holding one grid (equivalent to a batch of one). */
 crash_status crash_init_grid(const crash_grid_desc* desc, crash_ctx** out);

@@ -805,6 +805,62 @@ static int pass_crossings(const crash_ctx* c) {
   return most <= (int64_t)1 << 25 ? kLongPass : most <= (int64_t)1 << 26 ? 48 : 32;
 }
 
+// Device bytes of a workspace (its two record buffers, the packets' keys, ranks
+// and places, the bundles' direction keys).
+static size_t workspace_bytes(const WFSize& n, int nb) {
+  return (size_t)n.queue * (size_t)(2 * (((32 + 4 * nb) + 15) / 16 * 16)) + 12 * (size_t)std::max(n.queue, n.bundle) +
+         8 * (size_t)n.bundle_keys;
+}
+static std::string no_room(cudaError_t e) {
+  return e == cudaSuccess ? std::string("device memory cap (CRASH_DEVICE_MEMORY_CAP) exceeded by the packet queue")
+                          : std::string("packet workspace: ") + cudaGetErrorString(e);
+}
+
+// Makes sure that the context's workspace holds a step of `total` packets in
+// this form: the packet queue (two record buffers) or the sort buffers, sized
+// to the step (at most 2^28 packets per chunk: 38 GB of queue with 8 bins, 3.2
+// GB of sort buffers); nothing when every packet is traced to the end in
+// emission order.  It grows beside what earlier steps of the other form needed
+// (steps of both may alternate) or, if both have no room, in its place.  False
+// if this form alone has none: the cap (err is cudaSuccess; nothing changed) or
+// the device (err says why).
+static bool fit_workspace(crash_ctx* c, int form, int64_t total, cudaError_t* err) {
+  const int64_t chunk = c->opts.chunk_packets > 0 ? (int64_t)c->opts.chunk_packets : (int64_t)1 << 28;
+  const WFSize have = wavefront_size(c->wf);
+  WFSize want;
+  if (form == FORM_PASSES) {
+    want.queue = std::min<int64_t>(total, chunk);
+    want.n_keys = c->n_keys;
+  } else if (form == FORM_BUNDLE) {
+    want.bundle = std::min<int64_t>(total, chunk);
+    want.bundle_keys = std::max<int64_t>(c->n_src_total, std::min<int64_t>(kMaxBundleKeys, want.bundle / 2));
+  }
+  // (new sources may change the number of colours, and with it the length of a record)
+  if (c->wf && have.queue >= want.queue && have.bundle >= want.bundle && have.bundle_keys >= want.bundle_keys &&
+      (want.queue == 0 || have.nb == c->n_bins))
+    return true;
+  WFSize both;
+  both.queue = std::max(want.queue, have.queue);
+  both.n_keys = both.queue > 0 ? c->n_keys : 0;
+  both.bundle = std::max(want.bundle, have.bundle);
+  both.bundle_keys = std::max(want.bundle_keys, have.bundle_keys);
+  const size_t cap = memory_cap();
+  *err = cudaSuccess;
+  for (const WFSize& n : {both, want}) {
+    if (cap && c->bytes + workspace_bytes(n, c->n_bins) > cap) continue;
+    if (c->wf) {
+      cudaStreamSynchronize(c->stream);
+      wavefront_destroy(c->wf);
+      c->wf = nullptr;
+      if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
+    }
+    c->wf = wavefront_create(n, c->n_bins, err);
+    if (c->wf) return true;
+    cudaGetLastError();
+  }
+  return false;
+}
+
 extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t* P) {
   if (!c) return CRASH_ERR_ARG;
   if (!(dt > 0) || !isfinite(dt)) return set_err(c, CRASH_ERR_ARG, "dt must be positive");
@@ -850,61 +906,19 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
   }
   CK(cudaMemcpyAsync(c->d_meta, c->meta.data(), sizeof(BoxMeta) * c->n_boxes,
                      cudaMemcpyHostToDevice, c->stream));
-  int form = FORM_DIRECT;
-  int per_launch = 0;
+  int form = transport_form(c, total);
   {
-    // workspace: the packet queue (two record buffers) or the sort buffers
-    // of the step's form, sized to the step (at most 2^28 packets per chunk:
-    // 38 GB of queue with 8 bins, 3.2 GB of sort buffers); none when every
-    // packet is traced to the end in emission order.
-    form = transport_form(c, total);
-    per_launch = form == FORM_PASSES && !passes_asked(c->opts) ? pass_crossings(c) : 0;
-    const int64_t chunk = c->opts.chunk_packets > 0 ? (int64_t)c->opts.chunk_packets : (int64_t)1 << 28;
-    const WFSize have = wavefront_size(c->wf);
-    WFSize want;
-    if (form == FORM_PASSES) {
-      want.queue = std::min<int64_t>(total, chunk);
-      want.n_keys = c->n_keys;
-    } else if (form == FORM_BUNDLE) {
-      want.bundle = std::min<int64_t>(total, chunk);
-      want.bundle_keys = std::max<int64_t>(c->n_src_total, std::min<int64_t>(kMaxBundleKeys, want.bundle / 2));
-    }
-    // (new sources may change the number of colours, and with it the length of a record)
-    bool grow = !c->wf || have.queue < want.queue || have.bundle < want.bundle || have.bundle_keys < want.bundle_keys ||
-                (want.queue > 0 && have.nb != c->n_bins);
-    if (grow) {
-      want.queue = std::max(want.queue, have.queue);       // steps of both forms may alternate
-      want.n_keys = want.queue > 0 ? c->n_keys : 0;
-      want.bundle = std::max(want.bundle, have.bundle);
-      want.bundle_keys = std::max(want.bundle_keys, have.bundle_keys);
-      const size_t cap = memory_cap();
-      const size_t need = (size_t)want.queue * (size_t)(2 * (((32 + 4 * c->n_bins) + 15) / 16 * 16)) +
-                          12 * (size_t)std::max(want.queue, want.bundle) + 8 * (size_t)want.bundle_keys;
-      if (cap && c->bytes + need > cap) {
-        if (form != FORM_BUNDLE)
-          return set_err(c, CRASH_ERR_OOM, "device memory cap (CRASH_DEVICE_MEMORY_CAP) exceeded by the packet queue");
-        form = FORM_DIRECT;           // no room to sort: emission order needs none
-        want = WFSize();
-        grow = !c->wf;
-      }
-    }
-    if (grow) {
-      if (c->wf) {
-        CK(cudaStreamSynchronize(c->stream));
-        wavefront_destroy(c->wf);
-        c->wf = nullptr;
-        if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
-      }
-      cudaError_t e = cudaSuccess;
-      c->wf = wavefront_create(want, c->n_bins, &e);
-      if (!c->wf && form == FORM_BUNDLE) {
-        cudaGetLastError();
-        form = FORM_DIRECT;
-        c->wf = wavefront_create(WFSize(), c->n_bins, &e);
-      }
-      if (!c->wf) return set_err(c, CRASH_ERR_OOM, std::string("packet workspace: ") + cudaGetErrorString(e));
+    cudaError_t e = cudaSuccess;
+    if (!fit_workspace(c, form, total, &e)) {
+      // no room: passes that were asked for are refused; of the library's own
+      // forms bundles need less (12 bytes a packet) and emission order nothing
+      if (form == FORM_PASSES && passes_asked(c->opts)) return set_err(c, CRASH_ERR_OOM, no_room(e));
+      const bool bundles = form == FORM_PASSES && c->n_src_total <= kMaxBundleKeys && fit_workspace(c, FORM_BUNDLE, total, &e);
+      form = bundles ? FORM_BUNDLE : FORM_DIRECT;
+      if (!bundles && !fit_workspace(c, form, total, &e)) return set_err(c, CRASH_ERR_OOM, no_room(e));
     }
   }
+  const int per_launch = form == FORM_PASSES && !passes_asked(c->opts) ? pass_crossings(c) : 0;
   StepArgs a = make_args(c, dt, total);
   a.max_iter_step = step_max_iter;
   a.form = form;

@@ -1,5 +1,8 @@
 """The packet workspace a context keeps between steps: it is rebuilt when the
-sources' number of colours changes the length of a queue record."""
+sources' number of colours changes the length of a queue record; a step
+without room for it beside an earlier step's takes its place, and one without
+room for it alone runs in a form that needs less, unless passes were asked
+for."""
 import numpy as np
 import pytest
 
@@ -31,3 +34,45 @@ def test_new_sources_with_other_colours_in_passes(passes, order):
         for a, b in zip(_step(g, P, wavefront=0), got):
             assert np.array_equal(a, b), bins
     g.close()
+
+
+def test_passes_after_bundles_where_either_has_room(monkeypatch):
+    box = small_hhe_box((20, 20, 20), n_src=1, seed=781, thin=True)
+    ref, g = native.Grid(box, native.CRASH_MIXED), native.Grid(box, native.CRASH_MIXED)
+    # 0.7 MB of grid; the sort of 10^6 packets takes 16 MB, the queue of 10^5 14 MB
+    monkeypatch.setenv("CRASH_DEVICE_MEMORY_CAP", str(20_000_000))
+    for P, opts in [(1_000_000, {}), (100_000, dict(seg_per_iter=8)), (1_000_000, {}), (100_000, dict(seg_per_iter=8))]:
+        want = _step(ref, P, wavefront=0)
+        before = g.launch_count()
+        for a, b in zip(want, _step(g, P, **opts)):
+            assert np.array_equal(a, b), P
+        launches = g.launch_count() - before
+        assert launches == 7 if not opts else launches >= 4
+    g.close()
+    ref.close()
+
+
+@pytest.mark.parametrize("cap,launches", [(42_000_000, 3 + 4), (30_000_000, 3 + 1)])
+def test_passes_of_the_library_without_room(monkeypatch, cap, launches):
+    """Sources of few packets, for which the library takes passes (140 MB of
+    queue beside 22 MB of grid): bundles (16 MB) under one cap, emission order
+    under the other; passes asked for are refused, and nothing is lost by it."""
+    box = small_hhe_box((64, 64, 64), n_src=10_000, seed=782, thin=True)
+    P = 10_000 * 100
+    ref, g = native.Grid(box, native.CRASH_MIXED), native.Grid(box, native.CRASH_MIXED)
+    want = _step(ref, P, wavefront=0)
+    before = ref.launch_count()
+    _step(ref, P)
+    assert ref.launch_count() - before > 20          # (passes, where there is room)
+    monkeypatch.setenv("CRASH_DEVICE_MEMORY_CAP", str(cap))
+    before = g.launch_count()
+    for a, b in zip(want, _step(g, P)):
+        assert np.array_equal(a, b)
+    assert g.launch_count() - before == launches
+    with pytest.raises(native.CrashError) as e:
+        _step(g, P, seg_per_iter=32)
+    assert e.value.status == native.CRASH_ERR_OOM
+    for a, b in zip(want, _step(g, P)):
+        assert np.array_equal(a, b)
+    g.close()
+    ref.close()
