@@ -835,15 +835,19 @@ static bool fit_workspace(crash_ctx* c, int form, int64_t total, cudaError_t* er
     want.bundle = std::min<int64_t>(total, chunk);
     want.bundle_keys = std::max<int64_t>(c->n_src_total, std::min<int64_t>(kMaxBundleKeys, want.bundle / 2));
   }
+  // emission order asked for: the device gets the memory back
+  const bool give_back = c->precision == CRASH_MIXED && !c->opts.wavefront && (have.queue > 0 || have.bundle > 0);
   // (new sources may change the number of colours, and with it the length of a record)
-  if (c->wf && have.queue >= want.queue && have.bundle >= want.bundle && have.bundle_keys >= want.bundle_keys &&
+  if (!give_back && c->wf && have.queue >= want.queue && have.bundle >= want.bundle && have.bundle_keys >= want.bundle_keys &&
       (want.queue == 0 || have.nb == c->n_bins))
     return true;
-  WFSize both;
-  both.queue = std::max(want.queue, have.queue);
-  both.n_keys = both.queue > 0 ? c->n_keys : 0;
-  both.bundle = std::max(want.bundle, have.bundle);
-  both.bundle_keys = std::max(want.bundle_keys, have.bundle_keys);
+  WFSize both = want;
+  if (!give_back) {
+    both.queue = std::max(want.queue, have.queue);
+    both.n_keys = both.queue > 0 ? c->n_keys : 0;
+    both.bundle = std::max(want.bundle, have.bundle);
+    both.bundle_keys = std::max(want.bundle_keys, have.bundle_keys);
+  }
   const size_t cap = memory_cap();
   *err = cudaSuccess;
   for (const WFSize& n : {both, want}) {

@@ -2,7 +2,7 @@
 sources' number of colours changes the length of a queue record; a step
 without room for it beside an earlier step's takes its place, and one without
 room for it alone runs in a form that needs less, unless passes were asked
-for."""
+for; a step in emission order that was asked for gives it back."""
 import numpy as np
 import pytest
 
@@ -76,3 +76,17 @@ def test_passes_of_the_library_without_room(monkeypatch, cap, launches):
         assert np.array_equal(a, b)
     g.close()
     ref.close()
+
+
+def test_emission_order_gives_the_workspace_back():
+    torch = pytest.importorskip("torch")
+    box = small_hhe_box((16, 16, 16), n_src=2, seed=783)
+    g = native.Grid(box, native.CRASH_MIXED)
+    _step(g, 1000, wavefront=0)
+    g.sync()
+    free0 = torch.cuda.mem_get_info()[0]
+    _step(g, 2_000_000, seg_per_iter=64)             # a queue of 2e6 records: 280 MB
+    assert torch.cuda.mem_get_info()[0] < free0 - 200_000_000
+    _step(g, 1000, wavefront=0)
+    assert torch.cuda.mem_get_info()[0] > free0 - 50_000_000
+    g.close()
