@@ -264,8 +264,9 @@ int64_t crash_launch_count(crash_ctx* ctx);
    (opts.persistent); the state, the diffuse field's counts and the step
    index are restored afterwards.  Stores the fastest in the context's
    options (persistent included) and returns the chosen values (outputs may
-   be NULL).  The form the library chooses by itself (seg_per_iter and
-   resort_interval 0) is one of the trials. */
+   be NULL).  The form the library chooses by itself for the full step is one
+   of the trials, with the library's own blocks (block_size, seg_per_iter and
+   resort_interval 0). */
 crash_status crash_autotune(crash_ctx* ctx, double dt_s, const uint64_t* packets_per_box,
                             int* block_size, int* seg_per_iter, int* resort_interval,
                             int* reg_cap, int* tile, int* sort_curve);

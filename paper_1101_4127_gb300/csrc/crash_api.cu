@@ -865,7 +865,8 @@ static bool fit_workspace(crash_ctx* c, int form, int64_t total, cudaError_t* er
   return false;
 }
 
-extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t* P) {
+// One step; its form is that of a step of form_total packets (0: its own number).
+static crash_status step_batch(crash_ctx* c, double dt, const uint64_t* P, int64_t form_total) {
   if (!c) return CRASH_ERR_ARG;
   if (!(dt > 0) || !isfinite(dt)) return set_err(c, CRASH_ERR_ARG, "dt must be positive");
   if (!P) return set_err(c, CRASH_ERR_ARG, "packets_per_box is NULL");
@@ -910,7 +911,7 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
   }
   CK(cudaMemcpyAsync(c->d_meta, c->meta.data(), sizeof(BoxMeta) * c->n_boxes,
                      cudaMemcpyHostToDevice, c->stream));
-  int form = transport_form(c, total);
+  int form = transport_form(c, form_total > 0 ? form_total : total);
   {
     cudaError_t e = cudaSuccess;
     if (!fit_workspace(c, form, total, &e)) {
@@ -955,6 +956,10 @@ extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t
   c->chem_pending = !c->opts.chemistry;
   c->last_dt = dt;
   return CRASH_OK;
+}
+
+extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t* P) {
+  return step_batch(c, dt, P, 0);
 }
 
 extern "C" crash_status crash_step(crash_ctx* c, double dt, uint64_t P) {
@@ -1149,6 +1154,14 @@ extern "C" crash_status crash_autotune(crash_ctx* c, double dt, const uint64_t* 
                                        int* sort_curve) {
   if (!c || !P) return CRASH_ERR_ARG;
   cudaSetDevice(c->device);
+  // packets of the step that is tuned: trials trace fewer, in its form
+  int64_t full = 0;
+  for (int b = 0; b < c->n_boxes; ++b) {
+    if (!c->bh[b].has_sources) return set_err(c, CRASH_ERR_STATE, "a box has no sources");
+    const uint64_t n_src = (uint64_t)c->meta[b].n_src, Ns = P[b] / n_src;
+    const uint64_t lo = std::min<uint64_t>(c->opts.pkt_begin, Ns), hi = std::min<uint64_t>(c->opts.pkt_end, Ns);
+    full += (int64_t)(n_src * (hi > lo ? hi - lo : 0));
+  }
   // save the state and the step index so that trials leave no trace
   const size_t n = (size_t)c->n_cells;
   double* save = nullptr;
@@ -1199,7 +1212,7 @@ extern "C" crash_status crash_autotune(crash_ctx* c, double dt, const uint64_t* 
         for (int rs : resorts) trials.push_back({bs, sg, rs, cap, 0});
   if (c->precision == CRASH_MIXED) {
     trials.push_back({256, 0, 1, 0, 1});
-    trials.push_back({256, 0, 0, 0, 0});      // the form the library chooses by itself
+    trials.push_back({0, 0, 0, 0, 0});        // the form the library chooses by itself, with its own blocks
   }
   // the grid of trials runs one launch per pass; the fastest configuration is
   // then tried once more with Hilbert-ordered bucket keys, and the fastest of
@@ -1214,9 +1227,10 @@ extern "C" crash_status crash_autotune(crash_ctx* c, double dt, const uint64_t* 
     const Trial tr = ti >= n_grid ? Trial{best.block_size, best.seg_per_iter, best.resort_interval,
                                           best.reg_cap, best.tile}
                                   : trials[ti];
+    const bool own = tr.bs == 0;
     crash_run_opts o = base;
     o.sort_curve = curve_trial ? 1 : (pers_trial ? best.sort_curve : 0);
-    o.persistent = pers_trial ? 1 : 0;
+    o.persistent = pers_trial ? 1 : (own ? base.persistent : 0);
     o.block_size = tr.bs;
     o.seg_per_iter = tr.sg;
     o.resort_interval = tr.rs;
@@ -1231,10 +1245,10 @@ extern "C" crash_status crash_autotune(crash_ctx* c, double dt, const uint64_t* 
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    st = crash_step_batch(c, dt, P);                 // warm-up
+    st = step_batch(c, dt, P, full);                 // warm-up
     if (st == CRASH_OK) {
       cudaEventRecord(e0, c->stream);
-      st = crash_step_batch(c, dt, P);
+      st = step_batch(c, dt, P, full);
       cudaEventRecord(e1, c->stream);
     }
     cudaStreamSynchronize(c->stream);
