@@ -243,8 +243,11 @@ crash_status crash_checkpoint(crash_ctx* ctx, int op);
 crash_status crash_set_step_index(crash_ctx* ctx, uint64_t step);
 crash_status crash_sync(crash_ctx* ctx);
 
-/* Event-timed transport: total milliseconds and launch count of the dominant
-   transport kernel since the last reset (needs opts.timing = 1). */
+/* Event-timed transport: total milliseconds and number of the timed intervals
+   since the last reset (needs opts.timing = 1).  An interval is a launch that
+   emits or walks packets; in bundles it is a chunk, the sort by direction (which
+   draws the directions) and the walk together; in the FP64 form it is the
+   step's transport.  The sorts between passes are not in it. */
 crash_status crash_kernel_time(crash_ctx* ctx, double* ms_total, int64_t* launches);
 crash_status crash_reset_kernel_time(crash_ctx* ctx);
 

@@ -1679,9 +1679,9 @@ int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF
       const int64_t n = std::min<int64_t>(wf->bcap, a.total_packets - g0);
       WFArgs w = wf_args(wf, 0, true, false);
       w.work = wf->count + 2;
-      sort_bundles(a, wf, g0, n, s);
       const unsigned ntrace = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 4);
-      tic();
+      tic();                             // (the sort draws every direction: part of the emission)
+      sort_bundles(a, wf, g0, n, s);
       if (a.any_periodic) k_trace_bundle<NBT, HE, HEAT, true><<<ntrace, 256, 0, s>>>(a, t, w, g0, n, max_iter);
       else k_trace_bundle<NBT, HE, HEAT, false><<<ntrace, 256, 0, s>>>(a, t, w, g0, n, max_iter);
       toc();
