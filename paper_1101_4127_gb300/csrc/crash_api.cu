@@ -753,6 +753,13 @@ static bool passes_asked(const crash_run_opts& o) {
 // thousand packets on.
 constexpr int64_t kFp64Bundle = 8192;
 
+// cells of the largest box
+static int64_t largest_box(const crash_ctx* c) {
+  int64_t most = 0;
+  for (const BoxMeta& m : c->meta) most = std::max(most, m.ncell);
+  return most;
+}
+
 // Form of the transport of a step of `total` packets (the results do not
 // depend on it).
 static int transport_form(const crash_ctx* c, int64_t total) {
@@ -782,10 +789,9 @@ static int transport_form(const crash_ctx* c, int64_t total) {
   // 1.003 of the faster one's in the mean; none of 1, 3 or 16 colours (225
   // steps) is slower than before there were bundles.  (A batch counts as one
   // field: its packets are in flight in many boxes at once.)
-  int64_t most = 0;
-  for (const BoxMeta& m : c->meta) most = std::max(most, m.ncell);
+  const double most = (double)largest_box(c);
   const double per_source = (double)total / (double)c->n_src_total;
-  const double w = sqrt(32.0 * 3.14159265358979 * pow((double)most, 2.0 / 3.0) / per_source);
+  const double w = sqrt(32.0 * 3.14159265358979 * pow(most, 2.0 / 3.0) / per_source);
   const double fill = std::min(1.0, (double)total / (double)c->n_cells);
   const double narrow = (48 * c->n_cells > l2_bytes() ? 5.0 : 16.0) / sqrt(fill);
   if (w > narrow && total >= std::max<int64_t>(1 << 19, c->n_cells / 48)) return FORM_PASSES;
@@ -795,14 +801,26 @@ static int transport_form(const crash_ctx* c, int64_t total) {
 // the packets in flight spread, and the more cells a box has the farther the
 // absorbers and deposits they touch outgrow L2; short passes cost more queue
 // traffic and launches.  Thin fields, ms of a step's transport with passes of
-// 64 crossings in blocks of 128 with 64 registers / 48 in blocks of 256 with
-// 80 / 32 with 80: 1e8 packets, 256^3 177 / 191 / 198, 288^3 217 / 229 / 238,
-// 320^3 257 / 260 / 273, 384^3 383 / 319 / 333, 448^3 570 / 436 / 423, 512^3
-// 729 / 578 / 535; 2.5e8 packets, 512^3 1644 / 1258 / 1152.
+// 64 crossings with 64 registers in blocks of 128 | of 256 / 48 crossings with
+// 80 registers in blocks of 256 / 32 with 80: 1e8 packets, 256^3 177 | - / 191 /
+// 198, 288^3 217 | 216 / 229 / 238, 320^3 257 | 248 / 260 / 273, 384^3 383 | -
+// / 319 / 333, 448^3 570 | - / 436 / 423, 512^3 729 | - / 578 / 535; 2.5e8
+// packets, 512^3 1644 | - / 1258 / 1152.
 static int pass_crossings(const crash_ctx* c) {
-  int64_t most = 0;
-  for (const BoxMeta& m : c->meta) most = std::max(most, m.ncell);
+  const int64_t most = largest_box(c);
   return most <= (int64_t)1 << 25 ? kLongPass : most <= (int64_t)1 << 26 ? 48 : 32;
+}
+// Threads per block of the long passes.  Blocks of 128 wait less for their
+// slowest packet; in boxes that outgrow L2 by far blocks of 256, which take
+// their packets from one place in the order, are faster all the same.  ms for 128 / 256, thin, 20,000 sources, 1e7, 3e7 and 1e8 packets: 128^3
+// 11.2 / 11.4, 30.9 / 31.5, 99.1 / 100.9; 192^3 16.3 / 16.6, 44.9 / 45.7, 142 /
+// 144; 256^3 23.9 / 23.6, 60.6 / 61.0, 187 / 189; 288^3 32.8 / 30.8, 77.5 /
+// 73.9, 222 / 219; 320^3 41.7 / 38.8, 98.9 / 91.4, 272 / 259 (thick: 256^3 27.3
+// / 27.6, 72.9 / 74.1, 228 / 232; 320^3 42.6 / 40.4, 103.5 / 99.2, 296 / 295).
+// One colour walks faster and meets the line earlier: 192^3 13.1 / 13.5, 35.1 /
+// 36.2, 109.5 / 112.6; 256^3 23.1 / 21.6, 52.6 / 51.3, 151 / 153.
+static int pass_block(const crash_ctx* c) {
+  return largest_box(c) <= (int64_t)1 << (c->n_bins == 1 ? 23 : 24) ? 128 : 256;
 }
 
 // Device bytes of a workspace (its two record buffers, the packets' keys, ranks
@@ -928,6 +946,7 @@ static crash_status step_batch(crash_ctx* c, double dt, const uint64_t* P, int64
   a.max_iter_step = step_max_iter;
   a.form = form;
   a.launch_per_pass = per_launch;
+  a.pass_block = pass_block(c);
   const bool timing = c->opts.timing != 0;
   crash_status st;
   if (c->opts.use_graph && !timing) {

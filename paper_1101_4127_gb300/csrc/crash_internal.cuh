@@ -91,6 +91,7 @@ struct StepArgs {
   const BoxMeta* boxes_host;      // the same table in host memory (launch code only)
   int form;                       // mixed form: FORM_*
   int launch_per_pass;            // passes chosen by the library, one launch each: their crossings (0: as asked)
+  int pass_block;                 // threads per block of the long ones (launch_per_pass = kLongPass)
   int n_boxes;
   unsigned long long* step_dev;   // step index (Philox counter word), advanced on the device
   double dt;

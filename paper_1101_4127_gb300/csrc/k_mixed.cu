@@ -1635,10 +1635,9 @@ template <int NBT, bool HE, bool HEAT>
 int run_mixed(const StepArgs& a, const BinTables& t, const crash_run_opts& o, WF* wf, int max_iter,
               cudaStream_t s, EventPairs* ev, int* ev_used) {
   int launches = 0;
-  // (passes chosen by the library: blocks of 128 wait less for their slowest
-  // packet, 193.8 -> 190.5 ms on 1e8 packets of the thin 256^3 case)
+  // (the library's long passes have blocks and registers of their own)
   const bool long_passes = a.launch_per_pass == kLongPass;
-  const int block = o.block_size > 0 ? o.block_size : (long_passes ? 128 : 256);
+  const int block = o.block_size > 0 ? o.block_size : (long_passes ? a.pass_block : 256);
   const int persistent = num_sms() * (2048 / block);
   auto tic = [&]() {
     if (!ev) return;
