@@ -130,7 +130,9 @@ typedef struct {
   int chem_max_sub;          /* sub-step cap per cell and step (default 10000) */
   int cool_mask;             /* processes on: 1 coll. excitation, 2 coll. ionisation, 4 recombination,
                                 8 bremsstrahlung, 16 Compton, 32 dielectronic (default 63) */
-  int block_size;            /* threads per block of the transport kernels (0 = tuned/default) */
+  int block_size;            /* threads per block of the transport kernels in emission order and in
+                                passes, and of the FP64 form (0 = tuned/default); bundles of the
+                                mixed form and tile passes have blocks of their own */
   int seg_per_iter;          /* mixed form: crossings per packet per wavefront pass (0 = tuned) */
   int resort_interval;       /* mixed form: wavefront passes between Morton re-sorts (0 = tuned,
                                 <0 = never) */
@@ -139,13 +141,15 @@ typedef struct {
                                 resort_interval, pass_limit and tile all 0 it chooses by the
                                 step's sizes (emission order for few packets, bundles sorted by
                                 source and direction and traced to the end, or wavefront passes
-                                over a packet queue for large grids with many sources); any of
+                                over a packet queue for many packets from many sources); any of
                                 them nonzero asks for wavefront passes.  Results do not depend
                                 on it. */
   int use_graph;             /* 1: capture each step in a CUDA graph and replay it */
   int timing;                /* 1: record CUDA events around the transport launches */
-  int reg_cap;               /* mixed form: 1 = transport kernels capped at 64 registers
-                                (more resident warps), 0 = uncapped (tuned/default) */
+  int reg_cap;               /* mixed form, emission order and passes: 1 = transport kernels
+                                capped at 64 registers (more resident warps), 0 = uncapped
+                                (tuned/default; bundles, and the library's passes in boxes of
+                                up to 2^25 cells, are always capped) */
   int tile;                  /* mixed form: 1 = tile passes (packets sorted into 16^3-cell
                                 tiles; a tile's absorbers and deposits held in shared memory
                                 while its packets cross it); 0 = passes of seg_per_iter cells

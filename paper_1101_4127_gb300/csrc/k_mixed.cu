@@ -19,15 +19,16 @@
 //     stay within a few cells of one another: their gathers share sectors,
 //     their deposits in one cell are summed before they are sent, they take
 //     the same branches (thin or thick cells, which colours are left) and end
-//     together.  128^3, 1000 sources, 2e8 packets, 8 colours (1.61e10
-//     crossings): 244 ms against 383 ms for passes of the same walk;
+//     together.  128^3, 1000 sources, 2e8 packets, 8 colours (1.69e10
+//     crossings): a step's transport takes 225 ms, in passes of the same walk
+//     240 ms; with one source and 2e7 packets (thin) 17.0 and 25.7 ms;
 //   * passes (FORM_PASSES): the emission kernel writes every packet to a
 //     device queue; pass kernels (persistent, grid-stride over the live
 //     count held in device memory) advance the queue S steps at a time until
 //     it is empty.  Every R passes the queue is re-sorted by Morton order of
 //     its 8^3-cell bucket and direction (one-pass counting sort), so that the
-//     packets in flight, not only those of a warp, work on one part of a grid
-//     that does not fit L2.
+//     packets in flight, not only those of a warp, work on one part of the
+//     grid: for sources of so few packets that bundles are wide.
 // The launch sequence depends only on sizes and options, never on data,
 // so a step is capturable in a CUDA graph.
 #include <math.h>
