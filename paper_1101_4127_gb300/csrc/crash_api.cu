@@ -760,10 +760,39 @@ static int64_t largest_box(const crash_ctx* c) {
   return most;
 }
 
-// Form of the transport of a step of `total` packets (the results do not
-// depend on it).
-static int transport_form(const crash_ctx* c, int64_t total) {
+// What the form of a step is chosen by: its packets, the width of its bundles,
+// and the mean edge of the boxes (both as the packets' crossings see them:
+// weighted by packets times edge, and by packets).
+struct StepSizes {
+  int64_t total = 0;
+  double width = 0.0, edge = 0.0;
+};
+// of a step of P packets per box in the window [lo, hi) of ids (box sources set)
+static StepSizes step_sizes(const crash_ctx* c, const uint64_t* P, uint32_t lo, uint32_t hi) {
+  StepSizes z;
+  double paths = 0.0;
+  for (int b = 0; b < c->n_boxes; ++b) {
+    const BoxMeta& m = c->meta[b];
+    const uint64_t Ns = P[b] / (uint64_t)m.n_src;
+    const uint64_t l = std::min<uint64_t>(lo, Ns), h = std::min<uint64_t>(hi, Ns);
+    if (h <= l) continue;
+    const double n = cbrt((double)m.ncell), per_source = (double)(h - l), packets = per_source * m.n_src;
+    z.total += (int64_t)m.n_src * (int64_t)(h - l);
+    // 32 neighbouring directions of a source's, half the box away: w^2 = (n / 2)^2 4 pi 32 / (packets per source)
+    z.width += packets * n * (n * sqrt(32.0 * 3.14159265358979 / per_source));
+    paths += packets * n;
+  }
+  if (z.total > 0) {
+    z.width /= paths;
+    z.edge = paths / (double)z.total;
+  }
+  return z;
+}
+
+// Form of the transport of a step (the results do not depend on it).
+static int transport_form(const crash_ctx* c, const StepSizes& z) {
   const crash_run_opts& o = c->opts;
+  const int64_t total = z.total;
   if (c->precision != CRASH_MIXED)
     return total >= kFp64Bundle && c->n_src_total <= kMaxBundleKeys ? FORM_BUNDLE : FORM_DIRECT;
   if (!o.wavefront) return FORM_DIRECT;
@@ -772,29 +801,29 @@ static int transport_form(const crash_ctx* c, int64_t total) {
   if (total <= resident_packets()) return FORM_DIRECT;
   if (c->n_src_total > kMaxBundleKeys) return c->any_periodic ? FORM_DIRECT : FORM_PASSES;
   if (c->any_periodic) return FORM_BUNDLE;
-  // A bundle's 32 packets spread to about w cells at half the grid's width,
-  // w^2 = (n / 2)^2 4 pi 32 / (packets per source).  The wider the bundles, the
-  // less their lanes and their neighbours share of absorbers and deposits (48
-  // bytes a cell), and where these do not fit L2 they miss it too; passes in
-  // spatial order cost their sorts and win if there are packets enough to pay
-  // for these and to fill the buckets.  8 colours, thin, ms for bundles / passes
-  // (sources x packets per source, w): 128^3 300 x 67,000 (5) 19.9 / 20.4, 1000
-  // x 60,000 (5) 58.6 / 58.7, 10,000 x 600 (52) 9.5 / 7.0, 10^6 x 6 (524) 14.1 /
-  // 7.2; 160^3 300 x 67,000 (6) 27.6 / 25.4, 1000 x 60,000 (7) 82.6 / 71.7;
-  // 256^3 30 x 200,000 (6) 13.2 / 14.7, 300 x 200,000 (6) 138 / 116, 300 x 8,300
-  // (28) 12.6 / 9.6, 10^5 x 60 (331) 41.1 / 16.9; by number, 10^5 sources: 10^6
-  // packets 256^3 7.8 / 6.7, 320^3 10.7 / 10.4, 512^3 19.7 / 23.7; 512^3 2.5e6
-  // packets 43.4 / 44.1, 6e6 98.3 / 79.3.  Over 698 steps of 1 to 64 boxes, thin
-  // and thick, the rule's form takes 1.24 times the other's time at most and
-  // 1.003 of the faster one's in the mean; none of 1, 3 or 16 colours (225
-  // steps) is slower than before there were bundles.  (A batch counts as one
-  // field: its packets are in flight in many boxes at once.)
-  const double most = (double)largest_box(c);
-  const double per_source = (double)total / (double)c->n_src_total;
-  const double w = sqrt(32.0 * 3.14159265358979 * pow(most, 2.0 / 3.0) / per_source);
+  // A bundle's 32 packets spread to w cells half a box away.  The wider the
+  // bundles, the less their lanes and their neighbours share of absorbers and
+  // deposits (48 bytes a cell), and where a box's do not fit L2 they miss it
+  // too; passes in spatial order cost their sorts, as many as the largest box
+  // needs, and win if there are packets enough to pay for these and to fill the
+  // buckets.  8 colours, thin, ms for bundles / passes (sources x packets per
+  // source, w): 128^3 300 x 67,000 (5) 19.9 / 20.4, 1000 x 60,000 (5) 58.6 /
+  // 58.7, 10,000 x 600 (52) 9.5 / 7.0, 10^6 x 6 (524) 14.1 / 7.2; 160^3 300 x
+  // 67,000 (6) 27.6 / 25.4, 1000 x 60,000 (7) 82.6 / 71.7; 256^3 30 x 200,000 (6)
+  // 13.2 / 14.7, 300 x 200,000 (6) 138 / 116, 300 x 8,300 (28) 12.6 / 9.6, 10^5 x
+  // 60 (331) 41.1 / 16.9; by number, 10^5 sources: 10^6 packets 256^3 7.8 / 6.7,
+  // 320^3 10.7 / 10.4, 512^3 19.7 / 23.7; 512^3 2.5e6 packets 43.4 / 44.1, 6e6
+  // 98.3 / 79.3.  8 boxes of 128^3, 30,000 sources x 83 42 / 24, 300 x 25,000
+  // 62.6 / 61.4, 8 of 160^3, 300 x 25,000 100 / 84; 12 boxes of 32^3 to 128^3, 30
+  // sources x 16,666 4.2 / 4.8.  Over 1123 steps (1 to 64 boxes of one or several
+  // sizes, thin and thick, 1 to 16 colours) the rule's form takes 1.21 times the
+  // other's time at most and 1.004 times the faster one's in the mean, and none
+  // is slower than before there were bundles.
+  const double most = (double)largest_box(c), uneven = cbrt(most) / z.edge;
   const double fill = std::min(1.0, (double)total / (double)c->n_cells);
-  const double narrow = (48 * c->n_cells > l2_bytes() ? 5.0 : 16.0) / sqrt(fill);
-  if (w > narrow && total >= std::max<int64_t>(1 << 19, c->n_cells / 48)) return FORM_PASSES;
+  const double narrow = (48.0 * most > (double)l2_bytes() ? 5.0 : 16.0) / sqrt(fill);
+  const double least = std::max(524288.0, (double)c->n_cells / 48.0) * uneven * uneven;
+  if (z.width > narrow && (double)total >= least) return FORM_PASSES;
   return FORM_BUNDLE;
 }
 // Crossings per packet of the passes the library chooses.  Between two sorts
@@ -883,8 +912,8 @@ static bool fit_workspace(crash_ctx* c, int form, int64_t total, cudaError_t* er
   return false;
 }
 
-// One step; its form is that of a step of form_total packets (0: its own number).
-static crash_status step_batch(crash_ctx* c, double dt, const uint64_t* P, int64_t form_total) {
+// One step; its form is that of the step over the ids [form_lo, form_hi).
+static crash_status step_batch(crash_ctx* c, double dt, const uint64_t* P, uint32_t form_lo, uint32_t form_hi) {
   if (!c) return CRASH_ERR_ARG;
   if (!(dt > 0) || !isfinite(dt)) return set_err(c, CRASH_ERR_ARG, "dt must be positive");
   if (!P) return set_err(c, CRASH_ERR_ARG, "packets_per_box is NULL");
@@ -929,7 +958,7 @@ static crash_status step_batch(crash_ctx* c, double dt, const uint64_t* P, int64
   }
   CK(cudaMemcpyAsync(c->d_meta, c->meta.data(), sizeof(BoxMeta) * c->n_boxes,
                      cudaMemcpyHostToDevice, c->stream));
-  int form = transport_form(c, form_total > 0 ? form_total : total);
+  int form = transport_form(c, step_sizes(c, P, form_lo, form_hi));
   {
     cudaError_t e = cudaSuccess;
     if (!fit_workspace(c, form, total, &e)) {
@@ -978,7 +1007,7 @@ static crash_status step_batch(crash_ctx* c, double dt, const uint64_t* P, int64
 }
 
 extern "C" crash_status crash_step_batch(crash_ctx* c, double dt, const uint64_t* P) {
-  return step_batch(c, dt, P, 0);
+  return c ? step_batch(c, dt, P, c->opts.pkt_begin, c->opts.pkt_end) : CRASH_ERR_ARG;
 }
 
 extern "C" crash_status crash_step(crash_ctx* c, double dt, uint64_t P) {
@@ -1173,14 +1202,8 @@ extern "C" crash_status crash_autotune(crash_ctx* c, double dt, const uint64_t* 
                                        int* sort_curve) {
   if (!c || !P) return CRASH_ERR_ARG;
   cudaSetDevice(c->device);
-  // packets of the step that is tuned: trials trace fewer, in its form
-  int64_t full = 0;
-  for (int b = 0; b < c->n_boxes; ++b) {
+  for (int b = 0; b < c->n_boxes; ++b)
     if (!c->bh[b].has_sources) return set_err(c, CRASH_ERR_STATE, "a box has no sources");
-    const uint64_t n_src = (uint64_t)c->meta[b].n_src, Ns = P[b] / n_src;
-    const uint64_t lo = std::min<uint64_t>(c->opts.pkt_begin, Ns), hi = std::min<uint64_t>(c->opts.pkt_end, Ns);
-    full += (int64_t)(n_src * (hi > lo ? hi - lo : 0));
-  }
   // save the state and the step index so that trials leave no trace
   const size_t n = (size_t)c->n_cells;
   double* save = nullptr;
@@ -1264,10 +1287,10 @@ extern "C" crash_status crash_autotune(crash_ctx* c, double dt, const uint64_t* 
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    st = step_batch(c, dt, P, full);                 // warm-up
+    st = step_batch(c, dt, P, base.pkt_begin, base.pkt_end);   // warm-up (in the form of the step that is tuned)
     if (st == CRASH_OK) {
       cudaEventRecord(e0, c->stream);
-      st = step_batch(c, dt, P, full);
+      st = step_batch(c, dt, P, base.pkt_begin, base.pkt_end);
       cudaEventRecord(e1, c->stream);
     }
     cudaStreamSynchronize(c->stream);

@@ -21,6 +21,9 @@ def _box(n, n_src, seed):
                       bin_frac=np.tile(f, (n_src, 1)))
 
 
+SEVERAL = (32, 48, 64, 96, 128)
+
+
 @pytest.mark.parametrize("n,boxes,n_src,per_src,passes", [
     (256, 1, 100_000, 40, True),         # few packets per source, fewer than a quarter of the cells in all
     (128, 1, 100_000, 10, True),         # the same in a grid that fits L2
@@ -30,9 +33,12 @@ def _box(n, n_src, seed):
     (256, 1, 30, 30_000, False),         # 15, 22 at 0.054
     (128, 1, 10, 60_000, False),
     (64, 8, 5, 20_000, False),
+    (SEVERAL, 5, 30, 16_000, False),     # bundles 7 cells wide in the mean
+    (SEVERAL, 5, 3000, 400, True),       # 45
+    (SEVERAL, 5, 300, 800, False),       # 32, but few packets for the passes the largest box needs
 ])
 def test_form_by_sizes(n, boxes, n_src, per_src, passes):
-    batch = [_box(n, n_src, 820 + b) for b in range(boxes)]
+    batch = [_box(n if isinstance(n, int) else n[b], n_src, 820 + b) for b in range(boxes)]
     out = []
     for opts in ({}, dict(wavefront=0)):
         g = native.Grid(batch, native.CRASH_MIXED)
