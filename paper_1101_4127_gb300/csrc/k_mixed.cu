@@ -648,7 +648,7 @@ __device__ __forceinline__ int walk_steps(const bool run, int& ix, int& iy, int&
                  stz = dz > 0.f ? cells.nz : 0u - cells.nz;
   unsigned next = 0;
   float4 ab = make_float4(0.f, 0.f, 0.f, 0.f);
-  bool go = run, cut = false;
+  bool go = run, cut = false, spent = false;
   if (go) {
     next = cells.index(ix, iy, iz);
     ab = cells.load(next);
@@ -697,12 +697,16 @@ __device__ __forceinline__ int walk_steps(const bool run, int& ix, int& iy, int&
     // absorbs nothing and is no crossing)
     cell_attenuate<NBT, HE, HEAT>(seg, dl, here, N, nb, t, left, cells, cell, heat_box);
     tl.crossings += seg > 0.f ? 1u : 0u;
-    if (left == 0 && seg > 0.f) go = false;
+    if (left == 0 && seg > 0.f) {
+      go = false;
+      spent = true;
+    }
   }
   ix = dx > 0.f ? R.x1 - rx : R.x0 + rx - 1;
   iy = dy > 0.f ? R.y1 - ry : R.y0 + ry - 1;
   iz = dz > 0.f ? R.z1 - rz : R.z0 + rz - 1;
-  if (left == 0) return ABSORBED;
+  // (a packet without photons has made no crossing until a segment has a length)
+  if (spent) return ABSORBED;
   const bool out = ((unsigned)ix >= (unsigned)M->nx) | ((unsigned)iy >= (unsigned)M->ny) | ((unsigned)iz >= (unsigned)M->nz);
   return out || (PER && cut) ? ESCAPED : ALIVE;
 }

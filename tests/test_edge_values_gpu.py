@@ -123,3 +123,28 @@ def test_fp64_he_absorbers_that_are_not_numbers():
         g.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("bins", [1, 5, 8])
+def test_crossings_of_packets_without_photons(bins):
+    """A source of no luminosity on a cell's corner: its packets cross one cell,
+    after up to three segments of no length, whatever the pass length."""
+    box = small_hhe_box((17, 12, 16), n_src=2, seed=814, thin=True)
+    box.src_pos = np.array([[11.0, 3.0, 7.0], [6.5, 0.2, 15.1]])
+    box.src_ndot = np.array([0.0, 1e48])
+    box.bin_eV, box.bin_frac = _bins(bins), np.full((2, bins), 1.0 / bins)
+    P = 2 * 60_000
+    budgets = []
+    for opts in (dict(wavefront=0), dict(), dict(seg_per_iter=1), dict(seg_per_iter=2, persistent=0), dict(seg_per_iter=3),
+                 dict(seg_per_iter=64), dict(tile=1)):
+        g = native.Grid(box, native.CRASH_MIXED)
+        g.set_options(chemistry=0, **opts)
+        g.step(DT, P)
+        budgets.append(g.read(native.F_BUDGET)[:5].tolist())
+        g.close()
+    assert all(b == budgets[0] for b in budgets), budgets
+    g = native.Grid(box, native.CRASH_FP64_PLAIN)
+    g.set_options(chemistry=0)
+    g.step(DT, P)
+    assert g.read(native.F_BUDGET)[3] == budgets[0][3]
+    g.close()
