@@ -372,7 +372,8 @@ int or_freeze_absorbers(or_ctx* c) {
    photons (it leaves the step).  In each cell with path l > 0: per bin j,
    tau_j = l * sum_s n_s sigma_s,j; N' = rint(N exp(-tau_j)) (Eq. 1 in
    integer quanta); the absorbed A = N - N' goes to He I and He II by
-   rint(A kappa_s / kappa) and the rest to H I (Sec. 2 species split);
+   rint(A kappa_s / kappa) (0 where kappa is 0 or not a number) and the rest
+   to H I (Sec. 2 species split);
    the excess energy sum_s A_s (E_j - E_th,s) / 2^F is rounded once per
    cell.  Stops when every bin is empty or the packet leaves the grid. */
 int64_t or_trace_packet(or_ctx* c, const double pos[3], const double dir[3],
@@ -431,9 +432,11 @@ int64_t or_trace_packet(or_ctx* c, const double pos[3], const double dir[3],
         N[j] = Np;
         left |= Np;
         if (A > 0) {
-          int64_t A1 = llrint((double)A * (kHeI / kap));
+          /* (kap = 0 or not a number: no share, H I takes all) */
+          double f1 = kHeI / kap, f2 = kHeII / kap;
+          int64_t A1 = f1 == f1 ? llrint((double)A * f1) : 0;
           if (A1 > A) A1 = A;
-          int64_t A2 = llrint((double)A * (kHeII / kap));
+          int64_t A2 = f2 == f2 ? llrint((double)A * f2) : 0;
           if (A2 > A - A1) A2 = A - A1;
           int64_t A0 = A - A1 - A2;
           aHI += A0; aHeI += A1; aHeII += A2;

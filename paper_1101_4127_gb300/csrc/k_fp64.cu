@@ -240,14 +240,17 @@ __device__ __forceinline__ void walk_fp64(const StepArgs& a, const BinTables& t,
           long long A1 = 0, A2 = 0;
           const double Ad = (double)A;
           if (he1 || he2) {
-            // both shares over the one kappa
+            // both shares over the one kappa; where there is none (a cell without
+            // absorbers: A is then what the conversion of N to FP64 rounded off)
+            // or it is not a number, they are 0 and H I takes all
             const Divisor D(kap);
-            if (he1) {
-              A1 = llrint(Ad * D.of(kHeI));
+            const double f1 = D.of(kHeI), f2 = D.of(kHeII);
+            if (he1 && !not_a_number(f1)) {
+              A1 = llrint(Ad * f1);
               A1 = A1 > A ? A : A1;
             }
-            if (he2) {
-              A2 = llrint(Ad * D.of(kHeII));
+            if (he2 && !not_a_number(f2)) {
+              A2 = llrint(Ad * f2);
               A2 = A2 > A - A1 ? A - A1 : A2;
             }
           }

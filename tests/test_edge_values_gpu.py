@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 from paper_1101_4127_gb300 import inputs, native
-from _common import small_hhe_box
+from _common import assert_deposits_equal, pair, small_hhe_box
 
 pytestmark = pytest.mark.gpu
 DEPOSITS = [native.F_DEP_HI, native.F_DEP_HEI, native.F_DEP_HEII, native.F_DEP_E, native.F_BUDGET]
@@ -147,4 +147,29 @@ def test_crossings_of_packets_without_photons(bins):
     g.set_options(chemistry=0)
     g.step(DT, P)
     assert g.read(native.F_BUDGET)[3] == budgets[0][3]
+    g.close()
+
+
+@pytest.mark.parametrize("he,fractions", [(0.08, (1.0, 0.0, 1.0)), (0.08, (1.0, 0.0, 0.9)), (0.0, (1.0, 0.0, 0.0))])
+def test_fp64_cells_without_absorbers(he, fractions):
+    """FP64 form, cells with nothing left to absorb in some or all colours: what
+    rounding N to FP64 takes off goes to H I, and no deposit is out of range;
+    with He in the context (a pure-H box beside a box with He too), against the
+    oracle."""
+    boxes = [small_hhe_box((9, 8, 7), n_src=2, seed=815), small_hhe_box((6, 6, 6), n_src=1, seed=816)]
+    boxes[0].he_over_h = he
+    boxes[0].x_HII0, boxes[0].x_HeII0, boxes[0].x_HeIII0 = fractions
+    boxes[0].src_ndot = np.array([1.76e42, 5.2e42])
+    g = native.Grid(boxes, native.CRASH_FP64_PLAIN)
+    g.set_options(chemistry=0)
+    g.step(DT, [2 * 60, 700])
+    for i, box in enumerate(boxes):
+        _, o = pair(box)
+        o.set_options(chemistry=0)
+        o.step(DT, [2 * 60, 700][i])
+        assert_deposits_equal(g, o, i)
+        b = g.read(native.F_BUDGET, i)
+        assert b[0] == b[1] + b[2]
+        for f in DEPOSITS[:3]:
+            assert 0 <= g.read(f, i).min() and g.read(f, i).max() <= b[1]
     g.close()
